@@ -72,8 +72,7 @@ struct PatchHost {
     bool sat3_ok = false;             // every bucket fits the three-group kernel's row table
 };
 
-// A frame (or a scene's part of a frame) captured as CUDA graphs, one per
-// parity of the particle double buffers, with the pinned staging buffers
+// A frame captured as CUDA graphs, one per parity of the particle double buffers, with the pinned staging buffers
 // and the device block through which each replay gets its parameters.
 struct FrameGraph {
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
@@ -99,10 +98,6 @@ struct scwp_ctx {
     cudaStream_t st = nullptr;
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // particle-stage streams of a multi-patch context: patch i runs on
-    // pst[i % pst.size()], all forked from and joined back into st
-    std::vector<cudaStream_t> pst;
-    std::vector<cudaEvent_t> pev;
     std::string err;
     scwp_status sticky = SCWP_OK;
     SpectrumModel sm;
@@ -150,9 +145,9 @@ struct scwp_ctx {
     double b_makespan = 0.0;
     // captured batched frames (one per parity of the particle buffers)
     FrameGraph gfull;                 // whole batched frames (scwp_step)
-    FrameGraph gprep;                 // background + particle stages (the server's ticks)
     cudaStream_t gst = nullptr;       // capture origin (the caller's stream may be the legacy one)
     std::vector<InjectParams> ips;    // this frame's injection plans
+    std::vector<PatchDev> devs;       // the patches' descriptors as a launch takes them
     size_t alloc_bytes = 0;           // device memory held by the context
     unsigned int* queue = nullptr;    // work queue of the persistent summed-area synthesis (2 words)
     float* normal_scratch = nullptr;  // normals for host destinations
@@ -645,13 +640,6 @@ SynthParams synth_params(scwp_ctx* ctx, const PatchHost& P) {
     return sp;
 }
 
-scwp_status reset_frame_stats(scwp_ctx* ctx, PatchHost& P, cudaStream_t st) {
-    CU(cudaMemsetAsync(P.dev.stats, 0, 2 * sizeof(unsigned long long), st));
-    CU(cudaMemsetAsync(P.dev.stats + 3, 0, ((size_t)P.T.nb + 1) * sizeof(unsigned long long), st));
-    CU(cudaMemsetAsync(P.dev.stats + 5 + P.T.nb, 0, sizeof(unsigned long long), st));
-    return SCWP_OK;
-}
-
 // drop the captured frames (after a change that the captures baked in)
 void graph_reset(FrameGraph& G) {
     for (int k = 0; k < 2; ++k) {
@@ -664,28 +652,13 @@ void graph_reset(FrameGraph& G) {
     cudaGetLastError();
 }
 
-void graph_reset(scwp_ctx* ctx) {
-    graph_reset(ctx->gfull);
-    graph_reset(ctx->gprep);
-}
+void graph_reset(scwp_ctx* ctx) { graph_reset(ctx->gfull); }
 
-// streams for the particle stages of up to kParticleStreams patches at once
-constexpr int kParticleStreams = 8;
-scwp_status particle_streams(scwp_ctx* ctx) {
-    const size_t want = std::min<size_t>(ctx->patches.size(), kParticleStreams);
-    while (ctx->pst.size() < want) {
-        cudaStream_t s = nullptr;
-        cudaEvent_t e = nullptr;
-        if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-            if (s) cudaStreamDestroy(s);
-            cudaGetLastError();
-            return fail(ctx, SCWP_E_CUDA, "particle streams");
-        }
-        ctx->pst.push_back(s);
-        ctx->pev.push_back(e);
-    }
-    return SCWP_OK;
+// the patches' descriptors as of now, in patch order
+const PatchDev* patch_devs(scwp_ctx* ctx) {
+    ctx->devs.clear();
+    for (const PatchHost* P : ctx->patches) ctx->devs.push_back(P->dev);
+    return ctx->devs.data();
 }
 
 // device copies of the patch descriptors and synthesis parameters (and the
@@ -815,9 +788,7 @@ scwp_status scwp_create(const scwp_spectrum_desc* desc, scwp_ctx** out) {
         cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->gfull.done[0], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->gfull.done[1], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->gprep.done[0], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->gprep.done[1], cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&ctx->gfull.done[1], cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         return bail(SCWP_E_CUDA);
     }
@@ -912,7 +883,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
             P->bk[i].sat_c = amax[i] > 0 ? (float)(eps * 2147483648.0 / (0.6 * (double)amax[i])) : 3.0e38f;
     }
     const size_t cap = (size_t)D.cap;
-    D.nblk_c = (int)((cap + 1023) / 1024);
+    D.nblk_c = (int)((cap + kStepTile - 1) / kStepTile);
     D.nblk_s = (int)((2 * cap + kSortTile - 1) / kSortTile);
     D.nblk_o = (int)((2 * cap + kSortPassTile - 1) / kSortPassTile);
     bool ok = true;
@@ -924,8 +895,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
         D.vals[k] = (uint32_t*)dalloc(ctx, 2 * cap * 4);
         ok = ok && D.x[k] && D.y[k] && D.bd[k] && D.keys[k] && D.vals[k];
     }
-    D.count = (int32_t*)dalloc(ctx, 3 * sizeof(int32_t));
-    D.flags = (uint8_t*)dalloc(ctx, cap);
+    D.count = (int32_t*)dalloc(ctx, 2 * sizeof(int32_t));
     D.blk = (uint32_t*)dalloc(ctx, ((size_t)D.nblk_c + 1) * 4);
     const size_t ng = (size_t)T.nb * T.nth;
     D.vq = (int4*)dalloc(ctx, (ng + (D.emitter ? kWakeDirs : 0)) * sizeof(int4));
@@ -1004,8 +974,8 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
             ok = ok && D.partial;
         }
     }
-    D.stats = (unsigned long long*)dalloc(ctx, (6 + (size_t)T.nb) * sizeof(unsigned long long));
-    ok = ok && D.count && D.flags && D.blk && D.vq && D.dirlist && D.amp && D.bk && D.rot && D.phase && D.amax && D.hist &&
+    D.stats = (unsigned long long*)dalloc(ctx, stats_words(T.nb) * sizeof(unsigned long long));
+    ok = ok && D.count && D.blk && D.vq && D.dirlist && D.amp && D.bk && D.rot && D.phase && D.amax && D.hist &&
          D.offsets && D.rec && D.pk && D.out && D.stats;
     if (!ok) {
         delete P;
@@ -1044,7 +1014,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
     }
     int32_t n0 = (int32_t)std::min<size_t>(px.size(), cap);
     uint64_t flags0 = px.size() > cap ? kErrCapacity : 0;
-    int32_t counts[3] = {n0, n0, n0};
+    int32_t counts[2] = {n0, n0};
     CU(cudaMemcpyAsync(D.amp, ampf.data(), ng * sizeof(float), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(D.bk, P->bk.data(), T.nb * sizeof(BucketDev), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(P->d_items, P->tc_items.data(), P->tc_items.size() * sizeof(TcItem), cudaMemcpyHostToDevice,
@@ -1079,9 +1049,9 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
     }
     CU(cudaMemcpyAsync(D.phase, phase.data(), phase.size() * sizeof(float2), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(D.amax, amax.data(), amax.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->st));
-    CU(cudaMemsetAsync(D.flags, 0, cap, ctx->st));
+    CU(cudaMemsetAsync(D.blk, 0, ((size_t)D.nblk_c + 1) * 4, ctx->st));
     CU(cudaMemsetAsync(D.hist, 0, sort_words * 4, ctx->st));
-    CU(cudaMemsetAsync(D.stats, 0, (6 + (size_t)T.nb) * sizeof(unsigned long long), ctx->st));
+    CU(cudaMemsetAsync(D.stats, 0, stats_words(T.nb) * sizeof(unsigned long long), ctx->st));
     CU(cudaMemsetAsync(D.offsets, 0, ((size_t)D.total_bins + 1) * 4, ctx->st));
     CU(cudaMemsetAsync(D.out, 0, (size_t)3 * T.W * T.H * sizeof(float), ctx->st));
     if (n0 > 0) {
@@ -1261,6 +1231,7 @@ static void frame_injection(scwp_ctx* ctx, PatchHost* P, InjectParams& ip_out) {
         }
     }
     ip.nseg = nseg;
+    ip.given = given;
     ip.total = total;
     P->injected += total;
 }
@@ -1288,7 +1259,6 @@ static scwp_status enqueue_frame(scwp_ctx* ctx, const std::vector<InjectParams>&
         if ((s = record(ctx, fe->e[4], ctx->st)) != SCWP_OK) return s;
         CU(launch_background(ctx->bg, ctx->t, ctx->st, t_dev));
         if ((s = record(ctx, fe->e[5], ctx->st)) != SCWP_OK) return s;
-        CU(cudaEventRecord(ctx->ev_fork, ctx->st));   // the particle streams start after it
         CU(cudaEventRecord(ctx->ev_join, ctx->st));
     } else {
         CU(cudaEventRecord(ctx->ev_fork, ctx->st));
@@ -1298,31 +1268,19 @@ static scwp_status enqueue_frame(scwp_ctx* ctx, const std::vector<InjectParams>&
     }
     ctx->bg_valid = true;
 
-    // one patch: the context stream; several: up to kParticleStreams
-    // streams, so that the small kernels of different patches overlap
-    const bool multi = ctx->patches.size() > 1;
-    if (multi) {
-        if ((s = particle_streams(ctx)) != SCWP_OK) return s;
-        for (cudaStream_t ps : ctx->pst) CU(cudaStreamWaitEvent(ps, ctx->ev_fork, 0));
-    }
-    for (size_t k = 0; k < ctx->patches.size(); ++k) {
-        PatchHost* P = ctx->patches[k];
-        PatchDev& D = P->dev;
-        cudaStream_t pst = multi ? ctx->pst[P->index % ctx->pst.size()] : ctx->st;
-        CU(launch_advect_flag(D, pst));
-        CU(launch_compact(D, pst));
-        D.cur ^= 1;
+    // the particle stages, each one launch over all patches
+    const int np = (int)ctx->patches.size();
+    if (np > 0) {
+        const PatchDev* pd = patch_devs(ctx);
+        CU(launch_step(pd, np, ctx->st));
+        for (PatchHost* P : ctx->patches) P->dev.cur ^= 1;
+        pd = patch_devs(ctx);
         if (ip_dev)
-            CU(launch_inject_dev(D, ip_dev + k, pst));
-        else if (ips[k].total > 0)
-            CU(launch_inject(D, ips[k], pst));
-        CU(launch_bin(D, pst));   // (the frame's statistics were zeroed by the advection)
+            CU(launch_inject_dev(pd, ip_dev, np, ctx->st));
+        else
+            CU(launch_inject(pd, ips.data(), np, ctx->st));
+        CU(launch_bin(pd, np, false, ctx->st));
     }
-    if (multi)
-        for (size_t k = 0; k < ctx->pst.size(); ++k) {
-            CU(cudaEventRecord(ctx->pev[k], ctx->pst[k]));
-            CU(cudaStreamWaitEvent(ctx->st, ctx->pev[k], 0));
-        }
     if (fe && (s = record(ctx, fe->e[1], ctx->st)) != SCWP_OK) return s;
     CU(cudaStreamWaitEvent(ctx->st, ctx->ev_join, 0));
     if (fe && (s = record(ctx, fe->e[2], ctx->st)) != SCWP_OK) return s;
@@ -1332,39 +1290,14 @@ static scwp_status enqueue_frame(scwp_ctx* ctx, const std::vector<InjectParams>&
     return SCWP_OK;
 }
 
-// Background and particle stages of every patch of a scene, all on the
-// context stream (the server's ticks).  ips / ip_dev / t_dev as in
-// enqueue_frame.
-static scwp_status enqueue_prepare(scwp_ctx* ctx, const std::vector<InjectParams>& ips, const InjectParams* ip_dev,
-                                   const float2* t_dev) {
-    scwp_status s = SCWP_OK;
-    CU(launch_background(ctx->bg, ctx->t, ctx->st, t_dev));
-    ctx->bg_valid = true;
-    for (size_t k = 0; k < ctx->patches.size(); ++k) {
-        PatchHost* P = ctx->patches[k];
-        PatchDev& D = P->dev;
-        CU(launch_advect_flag(D, ctx->st));
-        CU(launch_compact(D, ctx->st));
-        D.cur ^= 1;
-        if (ip_dev)
-            CU(launch_inject_dev(D, ip_dev + k, ctx->st));
-        else if (ips[k].total > 0)
-            CU(launch_inject(D, ips[k], ctx->st));
-        CU(launch_bin(D, ctx->st));   // (the frame's statistics were zeroed by the advection)
-    }
-    CU(cudaGetLastError());
-    return SCWP_OK;
-}
-
-// Replay (capturing first if needed) graph set G with this frame's
-// parameters on `launch`.  A graph is captured once for each parity of the
+// Replay (capturing first if needed) graph set G, a whole frame, with this
+// frame's parameters on `launch`.  A graph is captured once for each parity of the
 // particle double buffers (every patch flips its live buffer each frame);
 // the frame's varying inputs (time, injection plans) reach it through one
 // copy from a pinned staging buffer per graph, rewritten only after that
-// graph's previous replay completed.  full: the whole frame (enqueue_frame);
-// otherwise the background and particle stages (enqueue_prepare).
+// graph's previous replay completed.
 static scwp_status run_graph(scwp_ctx* ctx, FrameGraph& G, const std::vector<InjectParams>& ips,
-                             cudaStream_t launch, bool full) {
+                             cudaStream_t launch) {
     scwp_status s = SCWP_OK;
     uint64_t mask = 0;
     for (size_t k = 0; k < ctx->patches.size(); ++k) mask |= (uint64_t)(ctx->patches[k]->dev.cur & 1) << k;
@@ -1399,10 +1332,7 @@ static scwp_status run_graph(scwp_ctx* ctx, FrameGraph& G, const std::vector<Inj
     memcpy(h + 16, ips.data(), ips.size() * sizeof(InjectParams));
     if (!G.valid[g]) {
         // everything that synchronises or allocates happens before the capture
-        if (full) {
-            if ((s = sync_synth(ctx)) != SCWP_OK) return s;
-            if (ctx->patches.size() > 1 && (s = particle_streams(ctx)) != SCWP_OK) return s;
-        }
+        if ((s = sync_synth(ctx)) != SCWP_OK) return s;
         if (!ctx->gst && cudaStreamCreateWithFlags(&ctx->gst, cudaStreamNonBlocking) != cudaSuccess) {
             ctx->gst = nullptr;
             return fail(ctx, SCWP_E_CUDA, "capture stream");
@@ -1418,8 +1348,7 @@ static scwp_status run_graph(scwp_ctx* ctx, FrameGraph& G, const std::vector<Inj
             e = cudaMemcpyAsync(G.dparams, h, bytes, cudaMemcpyHostToDevice, ctx->st);
             const InjectParams* ipd = reinterpret_cast<const InjectParams*>(G.dparams + 16);
             const float2* td = reinterpret_cast<const float2*>(G.dparams);
-            if (e == cudaSuccess)
-                s = full ? enqueue_frame(ctx, ips, ipd, td, nullptr) : enqueue_prepare(ctx, ips, ipd, td);
+            if (e == cudaSuccess) s = enqueue_frame(ctx, ips, ipd, td, nullptr);
             e2 = cudaStreamEndCapture(ctx->st, &graph);
         }
         ctx->st = caller;
@@ -1467,17 +1396,6 @@ static scwp_status frame_begin(scwp_ctx* ctx, double dt) {
     return SCWP_OK;
 }
 
-// A scene's frame up to the synthesis on `stream` (the server's ticks), as a
-// replayed graph.
-static scwp_status scene_prepare(scwp_ctx* ctx, double dt, cudaStream_t stream) {
-    cudaStream_t caller = ctx->st;
-    ctx->st = stream;
-    scwp_status s = frame_begin(ctx, dt);
-    ctx->st = caller;
-    if (s != SCWP_OK) return s;
-    return run_graph(ctx, ctx->gprep, ctx->ips, stream, false);
-}
-
 static scwp_status step_impl(scwp_ctx* ctx, double dt) {
     scwp_status s = frame_begin(ctx, dt);
     if (s != SCWP_OK) return s;
@@ -1489,7 +1407,7 @@ static scwp_status step_impl(scwp_ctx* ctx, double dt) {
     if (ctx->batched && !ctx->timing && ctx->patches.size() > 1 && ctx->patches.size() <= 64 &&
         (ctx->synth_mode == SCWP_SYNTH_GATHER || ctx->synth_mode == SCWP_SYNTH_GATHER_FP16 ||
          ctx->synth_mode == SCWP_SYNTH_SAT))
-        return run_graph(ctx, ctx->gfull, ctx->ips, ctx->st, true);
+        return run_graph(ctx, ctx->gfull, ctx->ips, ctx->st);
     FrameEvents* fe = nullptr;
     if (ctx->timing) {
         if (ctx->ring_n == kTimingRing && (s = drain_ring(ctx)) != SCWP_OK) return s;
@@ -1516,10 +1434,7 @@ scwp_status scwp_resynthesize(scwp_ctx* ctx, int32_t mode) {
         CU(launch_background(ctx->bg, ctx->t, ctx->st));
         ctx->bg_valid = true;
     }
-    for (PatchHost* P : ctx->patches) {
-        if ((s = reset_frame_stats(ctx, *P, ctx->st)) != SCWP_OK) return s;
-        CU(launch_bin(P->dev, ctx->st));
-    }
+    CU(launch_bin(patch_devs(ctx), (int)ctx->patches.size(), true, ctx->st));
     if ((s = synthesize(ctx, mode)) != SCWP_OK) return s;
     ctx->launches += launches_total() - before;
     CU(cudaStreamSynchronize(ctx->st));
@@ -2018,13 +1933,11 @@ void scwp_destroy(scwp_ctx* ctx) {
         cudaStreamSynchronize(ctx->st);
         if (ctx->side) cudaStreamSynchronize(ctx->side);
     }
-    for (cudaStream_t s : ctx->pst) cudaStreamSynchronize(s);
     graph_reset(ctx);
-    for (FrameGraph* G : {&ctx->gfull, &ctx->gprep})
-        for (int k = 0; k < 2; ++k) {
-            if (G->hstage[k]) cudaFreeHost(G->hstage[k]);
-            if (G->done[k]) cudaEventDestroy(G->done[k]);
-        }
+    for (int k = 0; k < 2; ++k) {
+        if (ctx->gfull.hstage[k]) cudaFreeHost(ctx->gfull.hstage[k]);
+        if (ctx->gfull.done[k]) cudaEventDestroy(ctx->gfull.done[k]);
+    }
     if (ctx->gst) cudaStreamDestroy(ctx->gst);
     cudaGetLastError();
     for (FrameEvents& f : ctx->ring)
@@ -2032,11 +1945,6 @@ void scwp_destroy(scwp_ctx* ctx) {
             if (f.e[k]) cudaEventDestroy(f.e[k]);
     for (PatchHost* P : ctx->patches) delete P;
     dfree_all(ctx);
-    for (cudaStream_t s : ctx->pst) {
-        cudaStreamSynchronize(s);
-        cudaStreamDestroy(s);
-    }
-    for (cudaEvent_t e : ctx->pev) cudaEventDestroy(e);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
     if (ctx->side) cudaStreamDestroy(ctx->side);
@@ -2048,10 +1956,11 @@ void scwp_destroy(scwp_ctx* ctx) {
 // =============================================================================
 // Frame-step server: continuous batching of frame-step requests over many
 // device-resident scenes (one context each).  A tick takes every idle scene
-// with a pending request, enqueues each one's background and particle stages
-// on one of eight streams, and runs the tensor-core synthesis of all of them
-// as one launch over the union of their batched-plan items (heaviest first)
-// on the server stream.  A scene has at most one frame in flight; at most
+// with a pending request, runs the background and particle stages of all of
+// them (each stage one launch over every patch of the tick, the backgrounds
+// of one grid size likewise, on a second stream), and their synthesis as one
+// launch over the union of their batched-plan items (heaviest first) on the
+// server stream.  A scene has at most one frame in flight; at most
 // `max_inflight` ticks are outstanding, so the next tick's particle stages
 // overlap the current tick's synthesis.  Scenes are admitted while their
 // device memory fits the budget.
@@ -2078,8 +1987,8 @@ struct ServerTick {
 struct scwp_server {
     scwp_server_desc d{};
     cudaStream_t st = nullptr;
-    std::vector<cudaStream_t> pst;
-    std::vector<cudaEvent_t> pev;
+    cudaStream_t pst[2] = {nullptr, nullptr};         // particle stages; backgrounds
+    cudaEvent_t pev[2] = {nullptr, nullptr};
     std::vector<ServerScene> scenes;
     std::deque<ServerTick> ticks;
     std::vector<cudaEvent_t> tick_events;             // one per staging slot
@@ -2145,14 +2054,9 @@ scwp_status scwp_server_create(const scwp_server_desc* desc, scwp_server** out) 
     bool ok = true;
     for (int k = 0; k < slots; ++k)
         ok = ok && cudaEventCreateWithFlags(&sv->tick_events[k], cudaEventDisableTiming) == cudaSuccess;
-    for (int k = 0; k < kParticleStreams && ok; ++k) {
-        cudaStream_t s = nullptr;
-        cudaEvent_t e = nullptr;
-        ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
-        if (s) sv->pst.push_back(s);
-        if (e) sv->pev.push_back(e);
-    }
+    for (int k = 0; k < 2 && ok; ++k)
+        ok = cudaStreamCreateWithFlags(&sv->pst[k], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&sv->pev[k], cudaEventDisableTiming) == cudaSuccess;
     if (ok) {
         sv->queue = (unsigned int*)sv_alloc(sv, 2 * sizeof(unsigned int));
         ok = sv->queue && cudaMemset(sv->queue, 0, 2 * sizeof(unsigned int)) == cudaSuccess;
@@ -2245,29 +2149,28 @@ scwp_status scwp_server_tick(scwp_server* sv, int32_t* started) {
     ServerTick tk;
     tk.slot = slot;
     tk.done = sv->tick_events[slot];
-    // background and particle stages, one scene per stream in turn
-    std::vector<bool> used(sv->pst.size(), false);
-    for (size_t k = 0; k < take.size(); ++k) {
-        ServerScene& sc = sv->scenes[take[k]];
-        const size_t q = k % sv->pst.size();
+    // the frames' host parts: times and injection plans (and, where dt
+    // changed, the tables, on the particle stream)
+    for (int i : take) {
+        ServerScene& sc = sv->scenes[i];
         const std::pair<int64_t, double> rq = sc.pending.front();
-        const scwp_status s = scene_prepare(sc.ctx, rq.second, sv->pst[q]);
+        cudaStream_t caller = sc.ctx->st;
+        sc.ctx->st = sv->pst[0];
+        const scwp_status s = frame_begin(sc.ctx, rq.second);
+        sc.ctx->st = caller;
         if (s != SCWP_OK) return sfail(sv, s, std::string("scene prepare: ") + sc.ctx->err);
-        used[q] = true;
         sc.pending.pop_front();
         sc.in_flight = true;
-        tk.reqs.emplace_back(take[k], rq.first);
+        tk.reqs.emplace_back(i, rq.first);
     }
-    for (size_t q = 0; q < sv->pst.size(); ++q)
-        if (used[q]) {
-            SCU(cudaEventRecord(sv->pev[q], sv->pst[q]));
-            SCU(cudaStreamWaitEvent(sv->st, sv->pev[q], 0));
-        }
     // the union of the scenes' synthesis plans, heaviest first: one list for
     // the scenes on the summed-area synthesis (the default), one for those on
     // the tensor-core gather
     std::vector<PatchDev> pd;
     std::vector<SynthParams> sp;
+    std::vector<InjectParams> ips;
+    std::vector<BgDev> bgs;
+    std::vector<double> bg_t;
     std::vector<TcItem> items[2];
     std::vector<double> work[2];
     std::vector<BlendSpan> spans[2];
@@ -2278,6 +2181,9 @@ scwp_status scwp_server_tick(scwp_server* sv, int32_t* started) {
             pd.push_back(c->patches[p]->dev);
             sp.push_back(c->h_sps[p]);
         }
+        ips.insert(ips.end(), c->ips.begin(), c->ips.end());
+        bgs.push_back(c->bg);
+        bg_t.push_back(c->t);
         const int m = c->synth_mode == SCWP_SYNTH_SAT ? 1 : 0;
         const std::vector<TcItem>& ci = m ? c->s_items : c->b_items;
         const std::vector<double>& cw = m ? c->s_work : c->b_work;
@@ -2305,7 +2211,8 @@ scwp_status scwp_server_tick(scwp_server* sv, int32_t* started) {
     o_bs[0] = o_it[0] + align16(items[0].size() * sizeof(TcItem));
     o_it[1] = o_bs[0] + align16(spans[0].size() * sizeof(BlendSpan));
     o_bs[1] = o_it[1] + align16(items[1].size() * sizeof(TcItem));
-    const size_t bytes = o_bs[1] + align16(std::max<size_t>(1, spans[1].size()) * sizeof(BlendSpan));
+    const size_t o_ip = o_bs[1] + align16(std::max<size_t>(1, spans[1].size()) * sizeof(BlendSpan));
+    const size_t bytes = o_ip + ips.size() * sizeof(InjectParams);
     if (sv->stage_cap[slot] < bytes) {
         if (sv->hstage[slot]) cudaFreeHost(sv->hstage[slot]);
         sv_free(sv, sv->dstage[slot]);
@@ -2330,8 +2237,26 @@ scwp_status scwp_server_tick(scwp_server* sv, int32_t* started) {
         for (size_t k = 0; k < order[m].size(); ++k) hi[k] = items[m][order[m][k]];
         if (!spans[m].empty()) memcpy(h + o_bs[m], spans[m].data(), spans[m].size() * sizeof(BlendSpan));
     }
+    memcpy(h + o_ip, ips.data(), ips.size() * sizeof(InjectParams));
     unsigned char* dv = (unsigned char*)sv->dstage[slot];
-    SCU(cudaMemcpyAsync(dv, h, bytes, cudaMemcpyHostToDevice, sv->st));
+    // the backgrounds, then the particle stages of every patch, beside each
+    // other on the tick streams; the synthesis waits for both
+    SCU(launch_backgrounds(bgs.data(), bg_t.data(), (int)bgs.size(), sv->pst[1]));
+    SCU(cudaMemcpyAsync(dv, h, bytes, cudaMemcpyHostToDevice, sv->pst[0]));
+    const int np = (int)pd.size();
+    SCU(launch_step(pd.data(), np, sv->pst[0]));
+    for (PatchDev& D : pd) D.cur ^= 1;
+    for (int i : take) {
+        scwp_ctx* c = sv->scenes[i].ctx;
+        c->bg_valid = true;
+        for (PatchHost* P : c->patches) P->dev.cur ^= 1;
+    }
+    SCU(launch_inject_dev(pd.data(), reinterpret_cast<const InjectParams*>(dv + o_ip), np, sv->pst[0]));
+    SCU(launch_bin(pd.data(), np, false, sv->pst[0]));
+    for (int q = 0; q < 2; ++q) {
+        SCU(cudaEventRecord(sv->pev[q], sv->pst[q]));
+        SCU(cudaStreamWaitEvent(sv->st, sv->pev[q], 0));
+    }
     const PatchDev* dpd = reinterpret_cast<const PatchDev*>(dv);
     const SynthParams* dsp = reinterpret_cast<const SynthParams*>(dv + o_sp);
     if (!items[0].empty())
@@ -2399,7 +2324,8 @@ const char* scwp_server_last_error(scwp_server* sv) { return sv ? sv->err.c_str(
 void scwp_server_destroy(scwp_server* sv) {
     if (!sv) return;
     if (sv->st) cudaStreamSynchronize(sv->st);
-    for (cudaStream_t s : sv->pst) cudaStreamSynchronize(s);
+    for (cudaStream_t s : sv->pst)
+        if (s) cudaStreamSynchronize(s);
     cudaGetLastError();
     for (ServerScene& sc : sv->scenes)
         if (sc.ctx) scwp_destroy(sc.ctx);
@@ -2410,8 +2336,10 @@ void scwp_server_destroy(scwp_server* sv) {
     for (cudaEvent_t e : sv->tick_events)
         if (e) cudaEventDestroy(e);
     sv_free(sv, sv->queue);
-    for (cudaStream_t s : sv->pst) cudaStreamDestroy(s);
-    for (cudaEvent_t e : sv->pev) cudaEventDestroy(e);
+    for (cudaStream_t s : sv->pst)
+        if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t e : sv->pev)
+        if (e) cudaEventDestroy(e);
     cudaGetLastError();
     delete sv;
 }

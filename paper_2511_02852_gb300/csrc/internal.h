@@ -8,6 +8,7 @@ namespace scwp {
 
 constexpr int kMaxBuckets = 64;
 constexpr int kRotN = 128;          // per-bucket phase-rotation table length
+constexpr int kStepTile = 1024;     // particles per tile of the step kernel
 constexpr int kSortTile = 1024;     // keys per block of the bin-key kernel
 constexpr int kSortPassTile = 4096; // keys per block of a binning sort pass
 constexpr int kMaxSortPasses = 4;   // 8-bit digits of keys up to 32 bits
@@ -51,9 +52,9 @@ struct PatchDev {
     int32_t* x[2] = {nullptr, nullptr};
     int32_t* y[2] = {nullptr, nullptr};
     uint32_t* bd[2] = {nullptr, nullptr}; // bucket << 16 | direction
-    int32_t* count = nullptr;             // [0] live, [1] live after compaction, [2] live before it
-    uint8_t* flags = nullptr;             // [cap] alive flags
-    uint32_t* blk = nullptr;              // [nblk_c + 1] compaction block sums
+    int32_t* count = nullptr;             // [0] live, [1] live after compaction
+    uint32_t* blk = nullptr;              // [nblk_c + 1] look-back words of the step's tiles, its ticket
+                                          // (zero between frames: the record pass clears them)
     int nblk_c = 0;
     int4* vq = nullptr;                   // [nb*nth (+4096)] (vx, vy, qx, qy)
     int16_t* dirlist = nullptr;           // [nb][2][nth] valid directions per edge pair
@@ -67,8 +68,8 @@ struct PatchDev {
     uint32_t* keys[2] = {nullptr, nullptr};  // [2 cap] bin keys (sort ping-pong)
     uint32_t* vals[2] = {nullptr, nullptr};  // [2 cap] bump ids
     // binning sort scratch (all zero between sorts: each pass's last block
-    // clears its histogram and ticket, the key kernel clears the look-back
-    // words before every sort)
+    // clears its histogram and ticket, the kernel that makes the keys clears
+    // the look-back words before every sort)
     uint32_t* hist = nullptr;             // [kMaxSortPasses][256] digit totals of each pass
     uint32_t* sort_ticket = nullptr;      // [kMaxSortPasses][2] block ticket, blocks done
     uint32_t* sort_status = nullptr;      // [kMaxSortPasses][nblk_o][256] look-back words
@@ -88,10 +89,17 @@ struct PatchDev {
                                           // [3+nb] operand stages of the last tensor-core synthesis,
                                           // [4+nb] evals summed over all frames,
                                           // [5+nb] candidates of the last summed-area synthesis
-                                          // (summed over its (tile, bucket) pairs)
+                                          // (summed over its (tile, bucket) pairs),
+                                          // then the frame's counts while its keys are made (stats_acc)
     float* layers = nullptr;              // layered variant scratch (lazy)
     size_t layers_bytes = 0;
 };
+
+// The counts of the frame whose keys are being made, zero between frames:
+// [0] evals, [1] binned, [2..2+nb) live per bucket.  The record pass, which
+// runs after every kernel that adds to them, publishes them in `stats`.
+__host__ __device__ inline unsigned long long* stats_acc(const PatchDev& p) { return p.stats + 6 + p.nb; }
+inline size_t stats_words(int nb) { return (size_t)(6 + nb) + (size_t)(2 + nb); }
 
 // One work item of the tensor-core synthesis: bucket group `group` of
 // `groups` over tile `tile` of patch `patch`.  The summed-area syntheses may
@@ -132,6 +140,7 @@ struct InjectParams {
     uint32_t patch;
     uint64_t seed;
     int W, H, nth;
+    int given;                // host-placed particles in use
     Segment seg[kMaxSegments];
     // wake (s = 2) and ring-ripple (s = 3) particles: Q16.16 positions and
     // wake-grid directions placed on the host in float64 (the operations that
@@ -202,13 +211,19 @@ inline int cached_per_device(int (&cache)[kMaxCachedDevices], F&& compute) {
 }
 
 // ---- launchers (each enqueues on `st`) --------------------------------------
-cudaError_t launch_advect_flag(const PatchDev& p, cudaStream_t st);
-cudaError_t launch_compact(const PatchDev& p, cudaStream_t st);
-cudaError_t launch_inject(const PatchDev& p, const InjectParams& ip, cudaStream_t st);
-// injection with the frame's parameters read from device memory (a fixed
-// grid, so that the launch can be replayed from a CUDA graph)
-cudaError_t launch_inject_dev(const PatchDev& p, const InjectParams* ip, cudaStream_t st);
-cudaError_t launch_bin(const PatchDev& p, cudaStream_t st);
+// The particle stages of n patches (ps: their descriptors, on the host),
+// each stage one launch over packs of up to 32 patches.
+// advection, expiry, compaction into the other buffer, and the survivors'
+// bin keys (the caller flips `cur` after it)
+cudaError_t launch_step(const PatchDev* ps, int n, cudaStream_t st);
+// injection (with keys), the frame's plans by value: patches with nothing to inject are
+// left out
+cudaError_t launch_inject(const PatchDev* ps, const InjectParams* ips, int n, cudaStream_t st);
+// injection with the frame's plans in device memory (a fixed grid, so that
+// the launch can be replayed from a CUDA graph)
+cudaError_t launch_inject_dev(const PatchDev* ps, const InjectParams* ips_dev, int n, cudaStream_t st);
+// the sort, offsets and records; keys: make the keys first (no step did)
+cudaError_t launch_bin(const PatchDev* ps, int n, bool keys, cudaStream_t st);
 // failure-detection self-test: the bin keys, then the first sort pass with
 // its first tile never taken, so the look-back waits on it give up after
 // wait_cycles SM clocks and set the timeout flag (outputs meaningless)
@@ -268,6 +283,9 @@ struct BgDev {
 // t_dev: if not null, the time is read from device memory (graph replay) as
 // a float pair (t_hi, t_lo), t = t_hi + t_lo, split on the host
 cudaError_t launch_background(const BgDev& b, double t, cudaStream_t st, const float2* t_dev = nullptr);
+// n backgrounds at their own times (a server's scenes): those of one grid
+// size share launches
+cudaError_t launch_backgrounds(const BgDev* b, const double* t, int n, cudaStream_t st);
 // complex elements of the row-pass intermediate of an N x N background
 size_t background_scratch_elems(int N);
 // entries of the twiddle tables of a length-N transform (at most N / 3)

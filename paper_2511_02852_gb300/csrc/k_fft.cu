@@ -261,13 +261,27 @@ __device__ __forceinline__ float phase(float2 w, float th, float tl) {
     return r + (e + c);
 }
 
+// The backgrounds of one launch (one grid size), blockIdx.y each: a server's
+// scenes step together, and one pair of launches each left the GPU idle
+// between them.
+constexpr int kBgMax = 16;
+template <int M>   // 1 or kBgMax
+struct BgPack {
+    static constexpr int kM = M;
+    BgDev b[M];
+    float th[M], tl[M];
+};
+
 // Rows pass: spectrum update (a1) + inverse FFT along x of H~, D~x, D~y for
 // row k_y = blockIdx.x in 0 .. N/2.  Block: 3 P threads; transform
 // f = tid / P.  h0 is [N][N] (FFT-natural order), omega [N][N] float pairs
 // (hi, lo); I is [3][N/2 + 1][N].
-template <int N>
+template <int N, int M>
 __global__ void __launch_bounds__(3 * threads_per_transform<N>(), N >= 4096 ? 1 : N >= 1024 ? 3 : 1)
-    k_spectrum_rows(BgDev bg, float th, float tl, const float2* t_dev) {
+    k_spectrum_rows(const __grid_constant__ BgPack<M> pk, const float2* t_dev) {
+    const int set = M == 1 ? 0 : blockIdx.y;
+    const BgDev& bg = pk.b[set];
+    float th = pk.th[set], tl = pk.tl[set];
     constexpr int P = threads_per_transform<N>(), Np = tstride<N>();
     constexpr int NT = 3 * P, E = (N + NT - 1) / NT;   // grid points per thread
     extern __shared__ float2 smem_rows[];
@@ -332,9 +346,11 @@ __global__ void __launch_bounds__(3 * threads_per_transform<N>(), N >= 4096 ? 1 
 // x0 .. x0 + 2 CZ - 1 of Dy (one transform W = Dy1(x) + i Dy1(x + 1) per
 // column pair).  The rows k_y > N/2 of H1, Dx1 and Dy1 are the conjugates of
 // the rows N - k_y.  out is [3][N][N] (h, Dx, Dy), row-major.
-template <int N>
+template <int N, int M>
 __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
-                                  col_group<N>() * threads_per_transform<N>() <= 512 ? 2 : 1) k_fft_cols(BgDev bg) {
+                                  col_group<N>() * threads_per_transform<N>() <= 512 ? 2 : 1)
+    k_fft_cols(const __grid_constant__ BgPack<M> pk) {
+    const BgDev& bg = pk.b[M == 1 ? 0 : blockIdx.y];
     constexpr int P = threads_per_transform<N>(), Np = tstride<N>(), CZ = col_group<N>();
     constexpr int NT = CZ * P;
     extern __shared__ float2 smem_cols[];
@@ -391,17 +407,17 @@ __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
     }
 }
 
-template <int N>
-cudaError_t launch_n(const BgDev& bg, float th, float tl, cudaStream_t st, const float2* t_dev) {
+template <int N, int M>
+cudaError_t launch_n(const BgPack<M>& pk, int m, cudaStream_t st, const float2* t_dev) {
     constexpr int P = threads_per_transform<N>(), CZ = col_group<N>();
     constexpr size_t smr = sizeof(float2) * 3 * tstride<N>(), smc = sizeof(float2) * CZ * tstride<N>();
     static_assert(smc <= 227 * 1024 && smr <= 227 * 1024, "shared memory of one CTA");
     static int attr[kMaxCachedDevices] = {};
     const int ok = cached_per_device(attr, [] {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_spectrum_rows<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
+            cudaFuncSetAttribute(k_spectrum_rows<N, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
         return (e == cudaSuccess &&
-                cudaFuncSetAttribute(k_fft_cols<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc) ==
+                cudaFuncSetAttribute(k_fft_cols<N, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc) ==
                     cudaSuccess)
                    ? 1
                    : -1;
@@ -411,32 +427,62 @@ cudaError_t launch_n(const BgDev& bg, float th, float tl, cudaStream_t st, const
         return cudaErrorInvalidValue;
     }
     cudaError_t e;
-    e = launch_pdl(k_spectrum_rows<N>, N / 2 + 1, 3 * P, smr, st, bg, th, tl, t_dev);
+    e = launch_pdl(k_spectrum_rows<N, M>, dim3(N / 2 + 1, m), 3 * P, smr, st, pk, t_dev);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_fft_cols<N>, N / CZ + N / (2 * CZ), CZ * P, smc, st, bg);
+    e = launch_pdl(k_fft_cols<N, M>, dim3(N / CZ + N / (2 * CZ), m), CZ * P, smc, st, pk);
     count_launches(2);
     return e;
+}
+
+template <int M>
+cudaError_t launch_pack(const BgPack<M>& pk, int m, cudaStream_t st, const float2* t_dev) {
+    switch (pk.b[0].N) {
+        case 8: return launch_n<8, M>(pk, m, st, t_dev);
+        case 16: return launch_n<16, M>(pk, m, st, t_dev);
+        case 32: return launch_n<32, M>(pk, m, st, t_dev);
+        case 64: return launch_n<64, M>(pk, m, st, t_dev);
+        case 128: return launch_n<128, M>(pk, m, st, t_dev);
+        case 256: return launch_n<256, M>(pk, m, st, t_dev);
+        case 512: return launch_n<512, M>(pk, m, st, t_dev);
+        case 1024: return launch_n<1024, M>(pk, m, st, t_dev);
+        case 2048: return launch_n<2048, M>(pk, m, st, t_dev);
+        case 4096: return launch_n<4096, M>(pk, m, st, t_dev);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// the time as a float pair (split on the host, in float64)
+template <int M>
+void pack_add(BgPack<M>& pk, int k, const BgDev& bg, double t) {
+    pk.b[k] = bg;
+    pk.th[k] = (float)t;
+    pk.tl[k] = (float)(t - (double)pk.th[k]);
 }
 
 }  // namespace
 
 cudaError_t launch_background(const BgDev& bg, double t, cudaStream_t st, const float2* t_dev) {
-    // the time as a float pair (split on the host, in float64)
-    const float th = (float)t;
-    const float tl = (float)(t - (double)th);
-    switch (bg.N) {
-        case 8: return launch_n<8>(bg, th, tl, st, t_dev);
-        case 16: return launch_n<16>(bg, th, tl, st, t_dev);
-        case 32: return launch_n<32>(bg, th, tl, st, t_dev);
-        case 64: return launch_n<64>(bg, th, tl, st, t_dev);
-        case 128: return launch_n<128>(bg, th, tl, st, t_dev);
-        case 256: return launch_n<256>(bg, th, tl, st, t_dev);
-        case 512: return launch_n<512>(bg, th, tl, st, t_dev);
-        case 1024: return launch_n<1024>(bg, th, tl, st, t_dev);
-        case 2048: return launch_n<2048>(bg, th, tl, st, t_dev);
-        case 4096: return launch_n<4096>(bg, th, tl, st, t_dev);
-        default: return cudaErrorInvalidValue;
+    BgPack<1> pk;
+    pack_add(pk, 0, bg, t);
+    return launch_pack(pk, 1, st, t_dev);
+}
+
+cudaError_t launch_backgrounds(const BgDev* b, const double* t, int n, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    for (int N = 8; N <= 4096 && e == cudaSuccess; N *= 2) {
+        BgPack<kBgMax> pk;
+        int m = 0;
+        for (int k = 0; k < n && e == cudaSuccess; ++k) {
+            if (b[k].N != N) continue;
+            pack_add(pk, m++, b[k], t[k]);
+            if (m == kBgMax) {
+                e = launch_pack(pk, m, st, nullptr);
+                m = 0;
+            }
+        }
+        if (m && e == cudaSuccess) e = launch_pack(pk, m, st, nullptr);
     }
+    return e;
 }
 
 size_t background_scratch_elems(int N) { return (size_t)3 * (N / 2 + 1) * N; }

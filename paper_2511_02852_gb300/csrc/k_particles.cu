@@ -1,6 +1,6 @@
 // Wave-particle state kernels of the hybrid ocean (sm_103a):
 //   advection + expiry + stable compaction  (Sec. 3.1 Lagrangian propagation,
-//                                            Sec. 4.1 WP updates),
+//     with the survivors' bin keys            Sec. 4.1 WP updates),
 //   boundary injection and wake emission     (Sec. 3.3 Eqs. 15-17, Sec. 4.3),
 //   per-bucket integer binning               (Sec. 4.2: the particles of a
 //                                            bucket share radius and kernel):
@@ -15,6 +15,8 @@
 
 #include <algorithm>
 #include <stdint.h>
+#include <string.h>
+#include <type_traits>
 
 #include "internal.h"
 #include "philox.h"
@@ -25,8 +27,24 @@ namespace {
 constexpr int kTpb = 256;
 constexpr int kItems = 4;                 // per thread in the compaction tiles
 constexpr int kTileC = kTpb * kItems;     // 1024 particles per compaction block
+static_assert(kTileC == kStepTile, "compaction words");
 constexpr int kTileS = kSortTile;     // keys per bin-key block
 constexpr int32_t kQi = 65536, kHalfi = 32768;
+
+// The patches of one launch, by value in the kernel's parameters (constant
+// bank: no load stands ahead of a block's first access).  Every particle
+// kernel runs over all patches of a frame at once, patch blockIdx.y, blocks
+// past a patch's own tiles returning at once: the stages of one patch are
+// short serial chains (4-7 us each on patches of up to 200k particles,
+// mostly latency), so one launch per patch and stage left the GPU nearly
+// idle and cost a launch each.  Packs of 1, 8 or 32 patches keep the
+// parameter copy near the patches there are (about 0.3 KB a patch).
+constexpr int kPackMax = 32;
+template <int M>
+struct PatchPack {
+    static constexpr int kM = M;
+    PatchDev p[M];
+};
 
 // Texel centres of [0, n) strictly inside (C - R, C + R) along one axis.
 __device__ __forceinline__ int span_count(int32_t C, int32_t R, int n) {
@@ -76,355 +94,13 @@ __device__ __forceinline__ float lookup_amp(const PatchDev& p, uint32_t bd) {
     return j < p.nth ? p.amp[b * p.nth + j] : p.wake_amp;
 }
 
-// Block-wide exclusive scan of one value per thread (kTpb threads).
-__device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t* s_warp, uint32_t& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t w = lane < kTpb / 32 ? s_warp[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        if (lane < kTpb / 32) s_warp[lane] = w;
-    }
-    __syncthreads();
-    total = s_warp[kTpb / 32 - 1];
-    const uint32_t before = warp ? s_warp[warp - 1] : 0u;
-    __syncthreads();
-    return before + x - v;
-}
+// 8-bit digits of a patch's bin keys
+__host__ __device__ __forceinline__ int sort_passes(const PatchDev& p) { return (p.key_bits + 7) / 8; }
 
-// ---- a3: advect, expire ------------------------------------------------------
-__global__ void __launch_bounds__(kTpb) k_advect_flag(PatchDev p) {
-    __shared__ uint32_t s_warp[kTpb / 32];
-    pdl_enter();
-    const int n = p.count[0];
-    if (blockIdx.x == 0) {
-        if (threadIdx.x == 0) p.count[2] = n;   // the pre-compaction count
-        // this frame's statistics start from zero (evals, binned, live per
-        // bucket, operand stages; the error flags stay)
-        if (threadIdx.x < 2) p.stats[threadIdx.x] = 0ull;
-        if (threadIdx.x <= p.nb) p.stats[3 + threadIdx.x] = 0ull;
-        if (threadIdx.x == 0) p.stats[5 + p.nb] = 0ull;
-    }
-    const int base = blockIdx.x * kTileC;
-    int32_t* X = p.x[p.cur];
-    int32_t* Y = p.y[p.cur];
-    const uint32_t* BD = p.bd[p.cur];
-    uint32_t alive_cnt = 0;
-    // the thread's kItems consecutive particles: one 16-byte access per array
-    // where all four are live (i0 is a multiple of 4)
-    static_assert(kItems == 4, "16-byte accesses of four particles");
-    const int i0 = base + threadIdx.x * kItems;
-    const bool full = i0 + kItems <= n;
-    int32_t xs[kItems], ys[kItems];
-    uint32_t bs[kItems];
-    if (full) {
-        const int4 a = *reinterpret_cast<const int4*>(X + i0);
-        const int4 b = *reinterpret_cast<const int4*>(Y + i0);
-        const uint4 c = *reinterpret_cast<const uint4*>(BD + i0);
-        xs[0] = a.x, xs[1] = a.y, xs[2] = a.z, xs[3] = a.w;
-        ys[0] = b.x, ys[1] = b.y, ys[2] = b.z, ys[3] = b.w;
-        bs[0] = c.x, bs[1] = c.y, bs[2] = c.z, bs[3] = c.w;
-    } else {
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            xs[k] = i0 + k < n ? X[i0 + k] : 0;
-            ys[k] = i0 + k < n ? Y[i0 + k] : 0;
-            bs[k] = i0 + k < n ? BD[i0 + k] : 0u;
-        }
-    }
-    uint32_t fl = 0u;   // the four alive flags, one byte each
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        if (i0 + k < n) {
-            const uint32_t bd = bs[k];
-            const int4 vq = lookup_vq(p, bd);
-            const int32_t x = xs[k] + vq.x, y = ys[k] + vq.y;
-            xs[k] = x;
-            ys[k] = y;
-            const int32_t R = p.bk[bd >> 16].R;
-            const bool a = (span_count(x, R, p.W) > 0 && span_count(y, R, p.H) > 0) ||
-                           (span_count(x - vq.z, R, p.W) > 0 && span_count(y - vq.w, R, p.H) > 0);
-            fl |= (a ? 1u : 0u) << (8 * k);
-            alive_cnt += a ? 1u : 0u;
-            if (!full) {
-                X[i0 + k] = x;
-                Y[i0 + k] = y;
-                p.flags[i0 + k] = a ? 1 : 0;
-            }
-        }
-    }
-    if (full) {
-        *reinterpret_cast<int4*>(X + i0) = make_int4(xs[0], xs[1], xs[2], xs[3]);
-        *reinterpret_cast<int4*>(Y + i0) = make_int4(ys[0], ys[1], ys[2], ys[3]);
-        *reinterpret_cast<uint32_t*>(p.flags + i0) = fl;
-    }
-    uint32_t total;
-    block_exscan(alive_cnt, s_warp, total);
-    if (threadIdx.x == 0) p.blk[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(kTpb) k_compact_scatter(PatchDev p) {
-    __shared__ uint32_t s_warp[kTpb / 32];
-    pdl_enter();
-    const int base = blockIdx.x * kTileC;
-    const int32_t* Xs = p.x[p.cur];
-    const int32_t* Ys = p.y[p.cur];
-    const uint32_t* Bs = p.bd[p.cur];
-    int32_t* Xd = p.x[1 - p.cur];
-    int32_t* Yd = p.y[1 - p.cur];
-    uint32_t* Bd = p.bd[1 - p.cur];
-    // only the pre-compaction live particles (count[2]) carry this frame's flags
-    const int n = p.count[2];
-    uint8_t f[kItems];
-    int32_t xs[kItems], ys[kItems];
-    uint32_t bs[kItems];
-    uint32_t mine = 0;
-    // every load first (one round trip): the earlier blocks' survivor
-    // counts, this tile's flags and particles (dead ones too: few)
-    uint32_t before = 0;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kTpb) before += p.blk[b];
-    const uint32_t blk_cnt = p.blk[blockIdx.x];
-    const int i0 = base + threadIdx.x * kItems;   // (a multiple of 4: 16-byte loads)
-    if (i0 + kItems <= n) {
-        const uint32_t fl = *reinterpret_cast<const uint32_t*>(p.flags + i0);
-        const int4 a = *reinterpret_cast<const int4*>(Xs + i0);
-        const int4 b = *reinterpret_cast<const int4*>(Ys + i0);
-        const uint4 c = *reinterpret_cast<const uint4*>(Bs + i0);
-        xs[0] = a.x, xs[1] = a.y, xs[2] = a.z, xs[3] = a.w;
-        ys[0] = b.x, ys[1] = b.y, ys[2] = b.z, ys[3] = b.w;
-        bs[0] = c.x, bs[1] = c.y, bs[2] = c.z, bs[3] = c.w;
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) f[k] = (uint8_t)((fl >> (8 * k)) & 0xFFu);
-    } else {
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            const int i = i0 + k;
-            f[k] = (i < n) ? p.flags[i] : 0;
-            xs[k] = (i < n) ? Xs[i] : 0;
-            ys[k] = (i < n) ? Ys[i] : 0;
-            bs[k] = (i < n) ? Bs[i] : 0u;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) mine += f[k];
-    // survivors of the earlier blocks, summed by this block (integers: any
-    // order); the last block also publishes the total as the new live count
-    uint32_t blk_off;
-    block_exscan(before, s_warp, blk_off);
-    if (blockIdx.x + 1 == (unsigned)p.nblk_c && threadIdx.x == 0) {
-        p.count[0] = (int32_t)(blk_off + blk_cnt);
-        p.count[1] = (int32_t)(blk_off + blk_cnt);
-    }
-    if (blk_cnt == 0) return;
-    uint32_t total;
-    uint32_t off = block_exscan(mine, s_warp, total) + blk_off;
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        if (f[k]) {
-            Xd[off] = xs[k];
-            Yd[off] = ys[k];
-            Bd[off] = bs[k];
-            ++off;
-        }
-    }
-}
-
-// ---- a4 + a5: injection and wake emission -------------------------------------
-__device__ __forceinline__ void inject_body(const PatchDev& p, const InjectParams& ip) {
-    const int base = p.count[1];
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const int64_t want = (int64_t)base + ip.total;
-        p.count[0] = (int32_t)(want > p.cap ? p.cap : want);
-        if (want > p.cap) atomicOr(&p.stats[2], (unsigned long long)kErrCapacity);
-    }
-    int32_t* X = p.x[p.cur];
-    int32_t* Y = p.y[p.cur];
-    uint32_t* BD = p.bd[p.cur];
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ip.total; e += gridDim.x * blockDim.x) {
-        const int64_t idx = (int64_t)base + e;
-        if (idx >= p.cap) break;
-        int sidx = 0;
-        while (sidx + 1 < ip.nseg && ip.seg[sidx + 1].first <= e) ++sidx;
-        const Segment sg = ip.seg[sidx];
-        const int le = e - sg.first;
-        int32_t x, y;
-        uint32_t bd;
-        if (sg.s < 2) {
-            const int g = le / sg.ndir, kk = le - g * sg.ndir;
-            const int j = p.dirlist[(sg.bucket * 2 + sg.s) * p.nth + kk];
-            const uint32_t ord = (uint32_t)(g * ip.nth + j);
-            const U4 u = philox4x32_10(ip.frame, ip.patch, (uint32_t)sg.bucket | ((uint32_t)sg.s << 16),
-                                       ord, ip.seed);
-            const int4 vq = p.vq[sg.bucket * p.nth + j];
-            const int32_t vn = sg.s == 0 ? vq.x : vq.y;
-            const uint64_t avn = (uint64_t)(vn < 0 ? -(int64_t)vn : (int64_t)vn);
-            const uint64_t len = (uint64_t)(sg.s == 0 ? ip.H : ip.W) * (uint64_t)kQi;
-            const int32_t along = (int32_t)(((uint64_t)u.x * len) >> 32);
-            const int32_t off = (int32_t)(((uint64_t)u.y * avn) >> 32);
-            const int32_t far = (sg.s == 0 ? ip.W : ip.H) * kQi;
-            const int32_t across = vn > 0 ? off : far - off;
-            x = sg.s == 0 ? across : along;
-            y = sg.s == 0 ? along : across;
-            bd = ((uint32_t)sg.bucket << 16) | (uint32_t)j;
-        } else {   // wake arms and ring ripples: positions placed on the host
-            const int gi = sg.given + le;
-            x = ip.gx[gi];
-            y = ip.gy[gi];
-            bd = ((uint32_t)sg.bucket << 16) | (uint32_t)(ip.nth + ip.ga[gi]);
-        }
-        X[idx] = x;
-        Y[idx] = y;
-        BD[idx] = bd;
-    }
-}
-
-__global__ void __launch_bounds__(kTpb) k_inject(PatchDev p, InjectParams ip) { pdl_enter(); inject_body(p, ip); }
-
-// the same with the frame's parameters in device memory (CUDA-graph replay)
-__global__ void __launch_bounds__(kTpb) k_inject_dev(PatchDev p, const InjectParams* ip) { pdl_enter(); inject_body(p, *ip); }
-
-// ---- a6: binning ---------------------------------------------------------------
-// Block b takes the particles of key tile b (kTileS / 2 particles, two bump
-// keys each) and adds the tile's counts of every sort pass's digit to the
-// passes' digit totals, so the passes need no histogram launch; block b also
-// clears the look-back words of sort-pass block b.
-__global__ void __launch_bounds__(kTpb) k_bin_keys(PatchDev p, uint32_t* keys, uint32_t* vals, int passes) {
-    __shared__ unsigned long long s_ev[kTpb / 32];
-    __shared__ unsigned int s_bin[kTpb / 32];
-    __shared__ unsigned int s_live[kMaxBuckets];
-    __shared__ uint32_t s_h[kMaxSortPasses][256];
-    static_assert(kTpb == 256, "one digit counter per thread");
-    pdl_enter();
-    for (int i = threadIdx.x; i < p.nb; i += blockDim.x) s_live[i] = 0;
-#pragma unroll
-    for (int ps = 0; ps < kMaxSortPasses; ++ps) s_h[ps][threadIdx.x] = 0;
-    if ((int)blockIdx.x < p.nblk_o)
-        for (int ps = 0; ps < passes; ++ps)
-            p.sort_status[((size_t)ps * p.nblk_o + blockIdx.x) * 256 + threadIdx.x] = 0u;
-    __syncthreads();
-    const int n = p.count[0];
-    const int32_t* X = p.x[p.cur];
-    const int32_t* Y = p.y[p.cur];
-    const uint32_t* BD = p.bd[p.cur];
-    unsigned long long ev = 0;
-    unsigned int binned = 0;
-    // the thread's kBinItems particles: every independent load first
-    constexpr int kBinItems = (kTileS / 2) / kTpb;
-    static_assert(kBinItems * kTpb == kTileS / 2, "whole particles per thread");
-    const int i0 = blockIdx.x * (kTileS / 2) + threadIdx.x;
-    uint32_t bd[kBinItems];
-    int32_t px[kBinItems], py[kBinItems];
-#pragma unroll
-    for (int m = 0; m < kBinItems; ++m) {
-        const int i = i0 + m * kTpb;
-        bd[m] = i < n ? BD[i] : 0u;
-        px[m] = i < n ? X[i] : 0;
-        py[m] = i < n ? Y[i] : 0;
-    }
-    // the state packed per particle for the record pass (one 16-byte gather
-    // per bump instead of three 4-byte ones)
-#pragma unroll
-    for (int m = 0; m < kBinItems; ++m) {
-        const int i = i0 + m * kTpb;
-        if (i < n) p.pk[i] = make_int4(px[m], py[m], (int)bd[m], 0);
-    }
-#pragma unroll
-    for (int m = 0; m < kBinItems; ++m) {
-        const int i = i0 + m * kTpb;
-        if (i >= n) continue;
-        const int b = (int)(bd[m] >> 16);
-        const int4 vq = lookup_vq(p, bd[m]);
-        const BucketDev bk = p.bk[b];
-        atomicAdd(&s_live[b], 1u);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int32_t cx = k ? px[m] - vq.z : px[m];
-            const int32_t cy = k ? py[m] - vq.w : py[m];
-            const int nx = span_count(cx, bk.R, p.W), ny = span_count(cy, bk.R, p.H);
-            uint32_t key = (uint32_t)p.total_bins;
-            if (nx > 0 && ny > 0) {
-                // (cx + R, cy + R > 0 here: the support reaches the patch)
-                int32_t rx, ry;
-                const int bx = floor_divmod(cx + bk.R, bk.C, rx);
-                const int by = floor_divmod(cy + bk.R, bk.C, ry);
-                key = (uint32_t)(bk.base + by * bk.nbx + bx);
-                ev += (unsigned long long)nx * (unsigned long long)ny;
-                ++binned;
-            }
-            keys[2 * i + k] = key;
-            vals[2 * i + k] = (uint32_t)(2 * i + k);
-            for (int ps = 0; ps < passes; ++ps) atomicAdd(&s_h[ps][(key >> (8 * ps)) & 255u], 1u);
-        }
-    }
-    // block reductions (integers: order-independent)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        ev += __shfl_down_sync(0xffffffffu, ev, o);
-        binned += __shfl_down_sync(0xffffffffu, binned, o);
-    }
-    if (lane == 0) {
-        s_ev[warp] = ev;
-        s_bin[warp] = binned;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long e = 0;
-        unsigned long long bb = 0;
-        for (int w = 0; w < kTpb / 32; ++w) {
-            e += s_ev[w];
-            bb += s_bin[w];
-        }
-        if (e) {
-            atomicAdd(&p.stats[0], e);
-            atomicAdd(&p.stats[4 + p.nb], e);   // running total over frames
-        }
-        if (bb) atomicAdd(&p.stats[1], bb);
-    }
-    for (int i = threadIdx.x; i < p.nb; i += blockDim.x)
-        if (s_live[i]) atomicAdd(&p.stats[3 + i], (unsigned long long)s_live[i]);
-    for (int ps = 0; ps < passes; ++ps)   // (after the barrier above)
-        if (s_h[ps][threadIdx.x]) atomicAdd(&p.hist[ps * 256 + threadIdx.x], s_h[ps][threadIdx.x]);
-}
-
-// ---- one LSD radix-sort pass (8-bit digit, stable) -----------------------------
-// Block-wide exclusive scan of one value per thread (kTpb threads); one
-// barrier inside, s_warp free on entry.
-__device__ __forceinline__ uint32_t block_exscan256(uint32_t v, uint32_t* s_warp) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[warp] = x;
-    __syncthreads();
-    uint32_t before = 0;
-#pragma unroll
-    for (int w = 0; w < kTpb / 32; ++w)
-        if (w < warp) before += s_warp[w];
-    return before + x - v;
-}
-
-constexpr int kPassItems = kSortPassTile / kTpb;   // keys per thread
-static_assert(kSortPassTile <= 65536, "tile ranks kept in 16 bits");
-constexpr int kPassWarpKeys = 32 * kPassItems;     // keys per warp: a contiguous run of the tile
 // look-back word: flag in the top two bits, a count below
 constexpr uint32_t kLbAggregate = 1u << 30, kLbPrefix = 2u << 30, kLbCount = (1u << 30) - 1u;
 constexpr long long kLbWaitCycles = 2000000000ll;  // the frame's limit: ~1 s at 2 GHz
 
-constexpr int kLbBatch = 8;                        // look-back words read per round trip
 // A look-back word carries its flag and count together, so plain relaxed
 // accesses (atomic per word, no ordering against other data) suffice, and
 // the loads of one batch overlap.
@@ -437,9 +113,412 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* a) {
     return v;
 }
 
+// ---- a6: bin keys -------------------------------------------------------------
+// A block's counts while it makes keys: every sort pass's digits (so the
+// passes need no histogram launch), live particles per bucket, evaluations
+// and binned bumps.
+struct KeyCounts {
+    uint32_t h[kMaxSortPasses][256];
+    unsigned int live[kMaxBuckets];
+    unsigned long long ev[kTpb / 32];
+    unsigned int bin[kTpb / 32];
+};
+static_assert(kTpb == 256, "one digit counter per thread");
+
+__device__ __forceinline__ void keys_begin(KeyCounts& C, const PatchDev& p) {   // (a block barrier must follow)
+    for (int i = threadIdx.x; i < p.nb; i += kTpb) C.live[i] = 0;
+#pragma unroll
+    for (int ps = 0; ps < kMaxSortPasses; ++ps) C.h[ps][threadIdx.x] = 0;
+}
+
+// block b of a kernel clears the look-back words of sort-pass block b
+__device__ __forceinline__ void clear_sort_words(const PatchDev& p) {
+    if ((int)blockIdx.x < p.nblk_o)
+        for (int ps = 0; ps < sort_passes(p); ++ps)
+            p.sort_status[((size_t)ps * p.nblk_o + blockIdx.x) * 256 + threadIdx.x] = 0u;
+}
+
+// Particle i of the patch (where `ok`; every lane of the warp calls): its
+// crest's and trough's keys, its state packed for the record pass (one
+// 16-byte gather per bump instead of three 4-byte ones), its counts.
+__device__ __forceinline__ void add_keys(KeyCounts& C, const PatchDev& p, int i, int32_t x, int32_t y, uint32_t bd,
+                                         int4 vq, bool ok, unsigned long long& ev, unsigned int& binned) {
+    const int b = (int)(bd >> 16);
+    // live particles per bucket, one shared atomic per bucket and warp
+    // (neighbours mostly share theirs: one per particle met 32 ways in
+    // one word)
+    const uint32_t peers = __match_any_sync(0xffffffffu, ok ? b : -1);
+    if (!ok) return;
+    if ((peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicAdd(&C.live[b], (unsigned)__popc(peers));
+    p.pk[i] = make_int4(x, y, (int)bd, 0);
+    const BucketDev bk = p.bk[b];
+    uint32_t key[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int32_t cx = k ? x - vq.z : x;
+        const int32_t cy = k ? y - vq.w : y;
+        const int nx = span_count(cx, bk.R, p.W), ny = span_count(cy, bk.R, p.H);
+        key[k] = (uint32_t)p.total_bins;
+        if (nx > 0 && ny > 0) {
+            // (cx + R, cy + R > 0 here: the support reaches the patch)
+            int32_t rx, ry;
+            const int bx = floor_divmod(cx + bk.R, bk.C, rx);
+            const int by = floor_divmod(cy + bk.R, bk.C, ry);
+            key[k] = (uint32_t)(bk.base + by * bk.nbx + bx);
+            ev += (unsigned long long)nx * (unsigned long long)ny;
+            ++binned;
+        }
+        for (int ps = 0; ps < sort_passes(p); ++ps) atomicAdd(&C.h[ps][(key[k] >> (8 * ps)) & 255u], 1u);
+    }
+    reinterpret_cast<uint2*>(p.keys[0])[i] = make_uint2(key[0], key[1]);
+}
+
+// The block's counts to the frame's (stats_acc, which the record pass
+// publishes and clears) and the passes' digit totals; every thread calls.
+__device__ __forceinline__ void keys_end(KeyCounts& C, const PatchDev& p, unsigned long long ev, unsigned int binned) {
+    // block reductions (integers: order-independent)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 16; o > 0; o >>= 1) {
+        ev += __shfl_down_sync(0xffffffffu, ev, o);
+        binned += __shfl_down_sync(0xffffffffu, binned, o);
+    }
+    if (lane == 0) {
+        C.ev[warp] = ev;
+        C.bin[warp] = binned;
+    }
+    __syncthreads();
+    unsigned long long* const acc = stats_acc(p);
+    if (threadIdx.x == 0) {
+        unsigned long long e = 0, bb = 0;
+        for (int w = 0; w < kTpb / 32; ++w) {
+            e += C.ev[w];
+            bb += C.bin[w];
+        }
+        if (e) atomicAdd(&acc[0], e);
+        if (bb) atomicAdd(&acc[1], bb);
+    }
+    for (int i = threadIdx.x; i < p.nb; i += kTpb)
+        if (C.live[i]) atomicAdd(&acc[2 + i], (unsigned long long)C.live[i]);
+    for (int ps = 0; ps < sort_passes(p); ++ps)   // (after the barrier above)
+        if (C.h[ps][threadIdx.x]) atomicAdd(&p.hist[ps * 256 + threadIdx.x], C.h[ps][threadIdx.x]);
+}
+
+// ---- a3: advect, expire, compact ------------------------------------------------
+// One pass over the state: a block takes tiles of 1024 particles in ticket
+// order, advects them, finds the survivors' new places by decoupled look-back
+// over the earlier tiles' counts (as the sort passes below do) and writes
+// them, with their bin keys, to the other buffer.  Separate launches for the
+// advection, the compaction and the keys moved 90 bytes a particle (the state
+// written and read back twice) and took three of a small frame's nine serial
+// launches; this moves 48 and is one.  The tile of the last particle
+// publishes the new count: by then every block with a tile has read the old
+// one, since that tile has seen all their counts.
+template <int M>
+__global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack<M> pk) {
+    __shared__ KeyCounts C;
+    __shared__ uint32_t s_cnt[32], s_off;   // survivors of 32-particle runs, then the runs' offsets
+    __shared__ int s_bid;
+    static_assert(kItems * kTpb / 32 == 32, "one run per lane of the scanning warp");
+    const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
+    pdl_enter();
+    if (M > 1 && (int)blockIdx.x >= p.nblk_c) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t* const words = p.blk;          // [nblk_c] look-back words, then the ticket
+    if (tid == 0) s_bid = (int)atomicAdd(words + p.nblk_c, 1u);
+    clear_sort_words(p);
+    keys_begin(C, p);
+    __syncthreads();
+    const int bid = s_bid;
+    const int n = p.count[0], base = bid * kTileC;
+    if (base >= n) {   // (uniform)
+        if (n == 0 && bid == 0 && tid == 0) p.count[1] = 0;
+        return;
+    }
+    const int32_t* X = p.x[p.cur];
+    const int32_t* Y = p.y[p.cur];
+    const uint32_t* BD = p.bd[p.cur];
+    int32_t xs[kItems], ys[kItems];
+    uint32_t bs[kItems], rank[kItems];
+    // particle of item k: base + k kTpb + tid; every load first
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        const int i = base + k * kTpb + tid;
+        bs[k] = i < n ? BD[i] : 0u;
+        xs[k] = i < n ? X[i] : 0;
+        ys[k] = i < n ? Y[i] : 0;
+    }
+    int4 vq[kItems];
+    uint32_t alive = 0u;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) vq[k] = lookup_vq(p, bs[k]);
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        const int i = base + k * kTpb + tid;
+        const int32_t x = xs[k] + vq[k].x, y = ys[k] + vq[k].y;
+        xs[k] = x;
+        ys[k] = y;
+        const int32_t R = p.bk[bs[k] >> 16].R;
+        const bool a = i < n && ((span_count(x, R, p.W) > 0 && span_count(y, R, p.H) > 0) ||
+                                 (span_count(x - vq[k].z, R, p.W) > 0 && span_count(y - vq[k].w, R, p.H) > 0));
+        const uint32_t m = __ballot_sync(0xffffffffu, a);
+        rank[k] = (uint32_t)__popc(m & ((1u << lane) - 1u));
+        alive |= (a ? 1u : 0u) << k;
+        if (lane == 0) s_cnt[k * (kTpb / 32) + warp] = (uint32_t)__popc(m);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t v = s_cnt[lane];
+        uint32_t inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        s_cnt[lane] = inc - v;
+        const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+        // survivors of the earlier tiles: 32 words at a time, back to the
+        // nearest inclusive prefix; an unpublished word is read again
+        uint32_t excl = 0;
+        if (bid > 0) {
+            if (lane == 0) st_relaxed(words + bid, kLbAggregate | total);
+            const long long t0 = clock64();
+            for (int j = bid - 1;;) {
+                const uint32_t w = j - lane >= 0 ? ld_relaxed(words + (j - lane)) : kLbPrefix;
+                const uint32_t pf = __ballot_sync(0xffffffffu, (w & ~kLbCount) == kLbPrefix);
+                const uint32_t un = __ballot_sync(0xffffffffu, (w & ~kLbCount) == 0u);
+                const int fp = pf ? __ffs(pf) - 1 : 32, fu = un ? __ffs(un) - 1 : 32;
+                const bool done = fp < fu;
+                const bool use = done ? lane <= fp : lane < fu;
+                excl += __reduce_add_sync(0xffffffffu, use ? w & kLbCount : 0u);
+                if (done) break;
+                j -= fu;
+                bool late = false;
+                if (lane == 0 && fu < 32) late = clock64() - t0 > kLbWaitCycles;
+                if (__any_sync(0xffffffffu, late)) {
+                    // (excl is then below the true offset: every store stays in bounds)
+                    if (lane == 0) atomicOr(&p.stats[2], (unsigned long long)kErrTimeout);
+                    break;
+                }
+            }
+        }
+        if (lane == 0) {
+            st_relaxed(words + bid, kLbPrefix | (excl + total));
+            s_off = excl;
+            if (base + kTileC >= n) p.count[0] = p.count[1] = (int32_t)(excl + total);
+        }
+    }
+    __syncthreads();
+    int32_t* Xd = p.x[1 - p.cur];
+    int32_t* Yd = p.y[1 - p.cur];
+    uint32_t* Bd = p.bd[1 - p.cur];
+    unsigned long long ev = 0;
+    unsigned int binned = 0;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        const int o = (int)(s_off + s_cnt[k * (kTpb / 32) + warp] + rank[k]);
+        const bool a = (alive >> k) & 1u;
+        if (a) {
+            Xd[o] = xs[k];
+            Yd[o] = ys[k];
+            Bd[o] = bs[k];
+        }
+        add_keys(C, p, o, xs[k], ys[k], bs[k], vq[k], a, ev, binned);
+    }
+    keys_end(C, p, ev, binned);
+}
+
+// ---- a4 + a5: injection and wake emission -------------------------------------
+// The injected particles follow the survivors, with their bin keys.  ip: the
+// frame's plan (InjectParams, or its InjectHead); seg, gx, gy, ga: its
+// segments and host-placed particles.
+template <typename IP>
+__device__ __forceinline__ void inject_body(const PatchDev& p, const IP& ip, const Segment* seg, const int32_t* gx,
+                                            const int32_t* gy, const int32_t* ga) {
+    __shared__ KeyCounts C;
+    const int base = p.count[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t want = (int64_t)base + ip.total;
+        p.count[0] = (int32_t)(want > p.cap ? p.cap : want);
+        if (want > p.cap) atomicOr(&p.stats[2], (unsigned long long)kErrCapacity);
+    }
+    if ((int)(blockIdx.x * kTpb) >= ip.total) return;   // (uniform)
+    keys_begin(C, p);
+    __syncthreads();
+    int32_t* X = p.x[p.cur];
+    int32_t* Y = p.y[p.cur];
+    uint32_t* BD = p.bd[p.cur];
+    unsigned long long ev = 0;
+    unsigned int binned = 0;
+    for (int e0 = blockIdx.x * kTpb; e0 < ip.total; e0 += gridDim.x * kTpb) {
+        const int e = e0 + threadIdx.x;
+        const int64_t idx = (int64_t)base + e;
+        const bool ok = e < ip.total && idx < p.cap;
+        int32_t x = 0, y = 0;
+        uint32_t bd = 0u;
+        if (ok) {
+            // the last segment that starts at or before e
+            int sidx = 0;
+            for (int hi = ip.nseg - 1; sidx < hi;) {
+                const int mid = (sidx + hi + 1) >> 1;
+                if (seg[mid].first <= e)
+                    sidx = mid;
+                else
+                    hi = mid - 1;
+            }
+            const Segment sg = seg[sidx];
+            const int le = e - sg.first;
+            if (sg.s < 2) {
+                const int g = le / sg.ndir, kk = le - g * sg.ndir;
+                const int j = p.dirlist[(sg.bucket * 2 + sg.s) * p.nth + kk];
+                const uint32_t ord = (uint32_t)(g * ip.nth + j);
+                const U4 u = philox4x32_10(ip.frame, ip.patch, (uint32_t)sg.bucket | ((uint32_t)sg.s << 16), ord,
+                                           ip.seed);
+                const int4 vq = p.vq[sg.bucket * p.nth + j];
+                const int32_t vn = sg.s == 0 ? vq.x : vq.y;
+                const uint64_t avn = (uint64_t)(vn < 0 ? -(int64_t)vn : (int64_t)vn);
+                const uint64_t len = (uint64_t)(sg.s == 0 ? ip.H : ip.W) * (uint64_t)kQi;
+                const int32_t along = (int32_t)(((uint64_t)u.x * len) >> 32);
+                const int32_t off = (int32_t)(((uint64_t)u.y * avn) >> 32);
+                const int32_t far = (sg.s == 0 ? ip.W : ip.H) * kQi;
+                const int32_t across = vn > 0 ? off : far - off;
+                x = sg.s == 0 ? across : along;
+                y = sg.s == 0 ? along : across;
+                bd = ((uint32_t)sg.bucket << 16) | (uint32_t)j;
+            } else {   // wake arms and ring ripples: positions placed on the host
+                const int gi = sg.given + le;
+                x = gx[gi];
+                y = gy[gi];
+                bd = ((uint32_t)sg.bucket << 16) | (uint32_t)(ip.nth + ga[gi]);
+            }
+            X[idx] = x;
+            Y[idx] = y;
+            BD[idx] = bd;
+        }
+        add_keys(C, p, (int)idx, x, y, bd, ok ? lookup_vq(p, bd) : make_int4(0, 0, 0, 0), ok, ev, binned);
+    }
+    keys_end(C, p, ev, binned);
+}
+
+// one patch, its plan by value
+__global__ void __launch_bounds__(kTpb) k_inject(const __grid_constant__ PatchDev p,
+                                                 const __grid_constant__ InjectParams ip) {
+    pdl_enter();
+    inject_body(p, ip, ip.seg, ip.gx, ip.gy, ip.ga);
+}
+
+// up to eight patches, their plans by value with only the segments and
+// placed particles in use (an InjectParams is 6.5 KB, a kernel's parameters
+// at most 32,764 bytes): patch k's segments start at word seg0[k] of `words`
+// and its placed particles (x, y, direction arrays of given[k]) at giv0[k]
+constexpr int kInjectMax = 8;
+constexpr int kInjectWords = 6400;   // 25,600 bytes: three patches with every segment in use
+struct InjectHead {
+    int nseg, total;
+    uint32_t frame, patch;
+    uint64_t seed;
+    int W, H, nth;
+};
+struct InjectPack {
+    PatchDev p[kInjectMax];
+    InjectHead h[kInjectMax];
+    int32_t seg0[kInjectMax], giv0[kInjectMax], given[kInjectMax];
+    uint32_t words[kInjectWords];
+};
+static_assert(sizeof(InjectPack) <= 32000, "kernel parameters");
+static_assert(sizeof(Segment) % 4 == 0, "segments in words");
+
+__global__ void __launch_bounds__(kTpb) k_inject_pack(const __grid_constant__ InjectPack pk) {
+    const int k = blockIdx.y;
+    pdl_enter();
+    const int32_t* g = reinterpret_cast<const int32_t*>(pk.words + pk.giv0[k]);
+    inject_body(pk.p[k], pk.h[k], reinterpret_cast<const Segment*>(pk.words + pk.seg0[k]), g, g + pk.given[k],
+                g + 2 * pk.given[k]);
+}
+
+// the frame's plans in device memory, one per patch (CUDA-graph replay and
+// the server's ticks)
+template <int M>
+__global__ void __launch_bounds__(kTpb) k_inject_dev(const __grid_constant__ PatchPack<M> pk, const InjectParams* ips) {
+    pdl_enter();
+    const InjectParams& ip = ips[blockIdx.y];
+    inject_body(pk.p[M == 1 ? 0 : blockIdx.y], ip, ip.seg, ip.gx, ip.gy, ip.ga);
+}
+
+// ---- a6: binning ---------------------------------------------------------------
+// The keys of a state as it stands (a resynthesis: no step made them).  Block
+// b takes the kTileS / 2 particles of key tile b.
+template <int M>
+__global__ void __launch_bounds__(kTpb) k_bin_keys(const __grid_constant__ PatchPack<M> pk) {
+    __shared__ KeyCounts C;
+    const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
+    pdl_enter();
+    if (M > 1 && (int)blockIdx.x >= p.nblk_s) return;
+    clear_sort_words(p);
+    const int n = p.count[0];
+    const int32_t* X = p.x[p.cur];
+    const int32_t* Y = p.y[p.cur];
+    const uint32_t* BD = p.bd[p.cur];
+    unsigned long long ev = 0;
+    unsigned int binned = 0;
+    // the thread's kBinItems particles: every independent load first
+    constexpr int kBinItems = (kTileS / 2) / kTpb;
+    static_assert(kBinItems * kTpb == kTileS / 2, "whole particles per thread");
+    const int b0 = blockIdx.x * (kTileS / 2), i0 = b0 + threadIdx.x;
+    if (b0 >= n) return;   // (uniform)
+    keys_begin(C, p);
+    uint32_t bd[kBinItems];
+    int32_t px[kBinItems], py[kBinItems];
+#pragma unroll
+    for (int m = 0; m < kBinItems; ++m) {
+        const int i = i0 + m * kTpb;
+        bd[m] = i < n ? BD[i] : 0u;
+        px[m] = i < n ? X[i] : 0;
+        py[m] = i < n ? Y[i] : 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < kBinItems; ++m) {
+        const int i = i0 + m * kTpb;
+        add_keys(C, p, i, px[m], py[m], bd[m], lookup_vq(p, bd[m]), i < n, ev, binned);
+    }
+    keys_end(C, p, ev, binned);
+}
+
+// ---- one LSD radix-sort pass (8-bit digit, stable) -----------------------------
+// A pass's block: 512 threads of 8 keys.  The ranking is a serial chain of one
+// round per key of a thread, so a tile's time goes with the keys per thread:
+// with 256 threads of 16 keys a pass over 4M keys took 42 us and one over a
+// single tile 9.6 us.
+constexpr int kSortTpb = 512;
+constexpr int kSortWarps = kSortTpb / 32;
+
+// Exclusive scan over the block's threads 0 .. 255 (v = 0 beyond them); one
+// barrier inside, s_warp free on entry.
+__device__ __forceinline__ uint32_t block_exscan256(uint32_t v, uint32_t* s_warp) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31 && warp < 8) s_warp[warp] = x;
+    __syncthreads();
+    uint32_t before = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w)
+        if (w < warp) before += s_warp[w];
+    return before + x - v;
+}
+
+constexpr int kPassItems = kSortPassTile / kSortTpb;   // keys per thread
+static_assert(kSortPassTile < 65536, "tile ranks and counts kept in 16 bits");
+constexpr int kPassWarpKeys = 32 * kPassItems;     // keys per warp: a contiguous run of the tile
+constexpr int kLbBatch = 8;                        // look-back words read per round trip
+
 // One pass: a persistent grid whose blocks take tiles of kSortPassTile keys
 // in ticket order.  A block ranks a tile's keys by digit (warp w holds the
-// tile's keys [512 w, 512 w + 512) in order, so ranks follow the input
+// tile's keys [256 w, 256 w + 256) in order, so ranks follow the input
 // order), publishes the tile's digit counts, and finds for each digit the
 // keys of that digit in the earlier tiles by looking back over their
 // published words (an inclusive prefix ends the walk) — the single-pass scan
@@ -456,28 +535,40 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* a) {
 // waits on it run out.  A block that gave up has summed a subset of the
 // earlier tiles' counts, so its output positions stay below the true ones
 // (in bounds, though the order is then wrong).
-__global__ void __launch_bounds__(kTpb, 3) k_sort_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
-                                                    uint32_t* vout, const int32_t* count, int shift,
-                                                    uint32_t* dtot, uint32_t* status, uint32_t* ticket,
-                                                    unsigned long long* err, long long wait_cycles,
-                                                    int first_tile) {
+// Pass ps of every patch of the pack that has so many digits (pass ps reads
+// key buffer ps & 1).  A patch's blocks share its own tickets, so its grid
+// may be any size.
+template <int M>
+__global__ void __launch_bounds__(kSortTpb, 3) k_sort_pass(const __grid_constant__ PatchPack<M> pk, int ps,
+                                                    long long wait_cycles, int first_tile) {
     __shared__ uint32_t s_k[kSortPassTile];
     __shared__ uint32_t s_v[kSortPassTile];
-    __shared__ uint32_t s_wh[kTpb / 32][256];   // per-warp digit counts, then the warp's offset in the digit
+    __shared__ uint16_t s_wh[kSortWarps][256];   // per-warp digit counts, then the warp's offset in the digit
     __shared__ uint32_t s_ls[256];              // the digit's first position in the reordered tile
     __shared__ uint32_t s_gb[256];              // output position of reordered tile position 0 of the digit
-    __shared__ uint32_t s_warp[kTpb / 32];
+    __shared__ uint32_t s_warp[8];
     __shared__ int s_bid;
     __shared__ bool s_last;
+    const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
+    if (M > 1 && ps >= sort_passes(p)) return;
+    const uint32_t* const kin = p.keys[ps & 1];
+    const uint32_t* const vin = p.vals[ps & 1];
+    uint32_t* const kout = p.keys[1 - (ps & 1)];
+    uint32_t* const vout = p.vals[1 - (ps & 1)];
+    const int shift = 8 * ps;
+    uint32_t* const dtot = p.hist + 256 * ps;
+    uint32_t* const status = p.sort_status + (size_t)ps * p.nblk_o * 256;
+    uint32_t* const ticket = p.sort_ticket + 2 * ps;
+    unsigned long long* const err = p.stats + 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = 2 * count[0];
-    const uint32_t gd = block_exscan256(dtot[tid], s_warp);   // keys of smaller digits, all tiles
+    const int n = 2 * p.count[0];
+    const uint32_t gd = block_exscan256(tid < 256 ? dtot[tid] : 0u, s_warp);   // keys of smaller digits, all tiles
     const uint32_t lt = (1u << lane) - 1u;
     for (;;) {
         if (tid == 0) s_bid = (int)atomicAdd(ticket, 1u) + first_tile;
 #pragma unroll
-        for (int w = 0; w < kTpb / 32; ++w) s_wh[w][tid] = 0u;
+        for (int w = tid; w < kSortWarps * 128; w += kSortTpb) reinterpret_cast<uint32_t*>(&s_wh[0][0])[w] = 0u;
         __syncthreads();   // (also: the previous tile's shared data is no longer read)
         const int bid = s_bid;
         const int base = bid * kSortPassTile;
@@ -490,7 +581,7 @@ __global__ void __launch_bounds__(kTpb, 3) k_sort_pass(const uint32_t* kin, cons
         for (int k = 0; k < kPassItems; ++k) {   // every load first
             const int i = i0 + 32 * k;
             kk[k] = i < n ? kin[i] : 0u;
-            vv[k] = i < n ? vin[i] : 0u;
+            vv[k] = ps == 0 ? (uint32_t)i : i < n ? vin[i] : 0u;   // (the keys come in bump order)
         }
 #pragma unroll
         for (int k = 0; k < kPassItems; ++k) {
@@ -501,58 +592,61 @@ __global__ void __launch_bounds__(kTpb, 3) k_sort_pass(const uint32_t* kin, cons
             const uint32_t before = act ? s_wh[warp][d] : 0u;
             rk[k / 2] |= (before + r) << (16 * (k & 1));
             __syncwarp();
-            if (act && r == 0) s_wh[warp][d] = before + __popc(peers);
+            if (act && r == 0) s_wh[warp][d] = (uint16_t)(before + __popc(peers));
             __syncwarp();
         }
         __syncthreads();
         // digit tid: each warp's offset within the tile's keys of the digit
-        uint32_t c = 0;
+        uint32_t c = 0, excl = 0;
+        if (tid < 256) {
 #pragma unroll
-        for (int w = 0; w < kTpb / 32; ++w) {
-            const uint32_t x = s_wh[w][tid];
-            s_wh[w][tid] = c;
-            c += x;
-        }
-        // keys of digit tid in the earlier tiles: walk back over their words,
-        // kLbBatch at a time, summing aggregates up to the nearest inclusive
-        // prefix; an unpublished word ends the batch and is read again
-        uint32_t excl = 0;
-        uint32_t* mine = status + (size_t)bid * 256 + tid;
-        if (bid == 0) {
-            st_relaxed(mine, kLbPrefix | c);
-        } else {
-            st_relaxed(mine, kLbAggregate | c);
-            const long long t0 = clock64();
-            int j = bid - 1;   // the nearest word not yet summed
-            for (;;) {
-                uint32_t w[kLbBatch];
+            for (int w = 0; w < kSortWarps; ++w) {
+                const uint32_t x = s_wh[w][tid];
+                s_wh[w][tid] = (uint16_t)c;
+                c += x;
+            }
+            // keys of digit tid in the earlier tiles: walk back over their words,
+            // kLbBatch at a time, summing aggregates up to the nearest inclusive
+            // prefix; an unpublished word ends the batch and is read again
+            uint32_t* mine = status + (size_t)bid * 256 + tid;
+            if (bid == 0) {
+                st_relaxed(mine, kLbPrefix | c);
+            } else {
+                st_relaxed(mine, kLbAggregate | c);
+                const long long t0 = clock64();
+                int j = bid - 1;   // the nearest word not yet summed
+                for (;;) {
+                    uint32_t w[kLbBatch];
 #pragma unroll
-                for (int q = 0; q < kLbBatch; ++q)
-                    w[q] = j - q >= 0 ? ld_relaxed(status + (size_t)(j - q) * 256 + tid) : kLbPrefix;
-                bool done = false, stalled = false;
+                    for (int q = 0; q < kLbBatch; ++q)
+                        w[q] = j - q >= 0 ? ld_relaxed(status + (size_t)(j - q) * 256 + tid) : kLbPrefix;
+                    bool done = false, stalled = false;
 #pragma unroll
-                for (int q = 0; q < kLbBatch; ++q) {
-                    if (done || stalled) continue;
-                    const uint32_t f = w[q] & ~kLbCount;
-                    if (f == 0u) {
-                        stalled = true;   // not yet published: read again from here
-                    } else {
-                        excl += w[q] & kLbCount;
-                        --j;
-                        done = f == kLbPrefix;
+                    for (int q = 0; q < kLbBatch; ++q) {
+                        if (done || stalled) continue;
+                        const uint32_t f = w[q] & ~kLbCount;
+                        if (f == 0u) {
+                            stalled = true;   // not yet published: read again from here
+                        } else {
+                            excl += w[q] & kLbCount;
+                            --j;
+                            done = f == kLbPrefix;
+                        }
+                    }
+                    if (done) break;
+                    if (stalled && clock64() - t0 > wait_cycles) {
+                        atomicOr(err, (unsigned long long)kErrTimeout);
+                        break;
                     }
                 }
-                if (done) break;
-                if (stalled && clock64() - t0 > wait_cycles) {
-                    atomicOr(err, (unsigned long long)kErrTimeout);
-                    break;
-                }
+                st_relaxed(mine, kLbPrefix | (excl + c));
             }
-            st_relaxed(mine, kLbPrefix | (excl + c));
         }
         const uint32_t ls = block_exscan256(c, s_warp);   // (its barrier orders s_wh above)
-        s_ls[tid] = ls;
-        s_gb[tid] = gd + excl - ls;
+        if (tid < 256) {
+            s_ls[tid] = ls;
+            s_gb[tid] = gd + excl - ls;
+        }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kPassItems; ++k) {
@@ -565,7 +659,7 @@ __global__ void __launch_bounds__(kTpb, 3) k_sort_pass(const uint32_t* kin, cons
         }
         __syncthreads();
         const int m = min(kSortPassTile, n - base);
-        for (int i = tid; i < m; i += kTpb) {
+        for (int i = tid; i < m; i += kSortTpb) {
             const uint32_t key = s_k[i];
             const uint32_t o = s_gb[(key >> shift) & 255u] + (uint32_t)i;
             kout[o] = key;
@@ -580,7 +674,7 @@ __global__ void __launch_bounds__(kTpb, 3) k_sort_pass(const uint32_t* kin, cons
     }
     __syncthreads();
     if (s_last) {
-        dtot[tid] = 0u;
+        if (tid < 256) dtot[tid] = 0u;
         if (tid == 0) {
             ticket[0] = 0u;
             ticket[1] = 0u;
@@ -593,7 +687,7 @@ int sort_pass_blocks_per_sm() {
     static int cache[kMaxCachedDevices];
     return cached_per_device(cache, [] {
         int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sort_pass, kTpb, 0) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sort_pass<1>, kSortTpb, 0) != cudaSuccess) {
             cudaGetLastError();
             return -1;
         }
@@ -622,11 +716,33 @@ int sm_count() {
 //    others sort last).
 constexpr int kRecItems = 4;   // sorted entries per thread and round, loads issued together
 
-__global__ void __launch_bounds__(kTpb) k_offsets_records(PatchDev p, const uint32_t* keys, const uint32_t* vals) {
+template <int M>
+__global__ void __launch_bounds__(kTpb) k_offsets_records(const __grid_constant__ PatchPack<M> pk) {
     // per warp: the 32 records of its 32 consecutive entries (1 KB), stored
     // out as 16-byte chunks of consecutive addresses (whole sectors)
     __shared__ uint4 s_rec[kTpb / 32][64];
+    const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
+    const uint32_t* const keys = p.keys[sort_passes(p) & 1];
+    const uint32_t* const vals = p.vals[sort_passes(p) & 1];
+    // the frame's statistics (the error flags stay; the synthesis counts its
+    // stages and candidates from zero), and the step's look-back words and
+    // ticket cleared for the next frame
+    if (blockIdx.x == 0) {
+        unsigned long long* const acc = stats_acc(p);
+        const int t = threadIdx.x;
+        if (t < 2) {
+            p.stats[t] = acc[t];
+            if (t == 0) p.stats[4 + p.nb] += acc[0];   // running total over frames
+            acc[t] = 0ull;
+        }
+        if (t < p.nb) {
+            p.stats[3 + t] = acc[2 + t];
+            acc[2 + t] = 0ull;
+        }
+        if (t == p.nb) p.stats[3 + p.nb] = p.stats[5 + p.nb] = 0ull;
+    }
+    for (int i = blockIdx.x * kTpb + threadIdx.x; i <= p.nblk_c; i += gridDim.x * kTpb) p.blk[i] = 0u;
     const int n = 2 * p.count[0];
     const int4* PK = p.pk;
     const uint32_t tb = (uint32_t)p.total_bins;
@@ -700,75 +816,139 @@ __global__ void __launch_bounds__(kTpb) k_offsets_records(PatchDev p, const uint
     }
 }
 
+// f(pack, patches in it) over packs of the n patches at ps
+template <typename F>
+cudaError_t for_packs(const PatchDev* ps, int n, F&& f) {
+    auto run = [&](auto tag, const PatchDev* q, int m) {
+        PatchPack<decltype(tag)::value> pk;
+        for (int k = 0; k < m; ++k) pk.p[k] = q[k];
+        return f(pk, m);
+    };
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < n && e == cudaSuccess; k += kPackMax) {
+        const int m = std::min(kPackMax, n - k);
+        e = m == 1   ? run(std::integral_constant<int, 1>(), ps + k, m)
+            : m <= 8 ? run(std::integral_constant<int, 8>(), ps + k, m)
+                     : run(std::integral_constant<int, kPackMax>(), ps + k, m);
+    }
+    return e;
+}
+
+template <typename PK, typename G>
+int pack_max(const PK& pk, int m, G&& g) {
+    int v = 1;
+    for (int k = 0; k < m; ++k) v = std::max(v, (int)g(pk.p[k]));
+    return v;
+}
+
+template <typename PK>
+cudaError_t launch_keys(const PK& pk, int m, cudaStream_t st) {
+    count_launches(1);
+    return launch_pdl(k_bin_keys<PK::kM>, dim3(pack_max(pk, m, [](const PatchDev& p) { return p.nblk_s; }), m), kTpb, 0,
+                      st, pk);
+}
+
+// a sort pass: up to the blocks that fit at once per patch (they take tiles
+// in turn)
+template <typename PK>
+cudaError_t launch_sort(const PK& pk, int m, int ps, long long wait_cycles, int first_tile, cudaStream_t st) {
+    const int fit = std::max(1, sort_pass_blocks_per_sm()) * std::max(1, sm_count());
+    const int grid = std::min(fit, pack_max(pk, m, [](const PatchDev& p) { return p.nblk_o; }));
+    count_launches(1);
+    return launch_pdl(k_sort_pass<PK::kM>, dim3(grid, m), kSortTpb, 0, st, pk, ps, wait_cycles, first_tile);
+}
+
 }  // namespace
 
 // ---- launchers -------------------------------------------------------------------
-cudaError_t launch_advect_flag(const PatchDev& p, cudaStream_t st) {
-    const cudaError_t e = launch_pdl(k_advect_flag, p.nblk_c, kTpb, 0, st, p);
-    count_launches(1);
-    return e;
+cudaError_t launch_step(const PatchDev* ps, int n, cudaStream_t st) {
+    return for_packs(ps, n, [&](const auto& pk, int m) {
+        constexpr int M = std::decay_t<decltype(pk)>::kM;
+        count_launches(1);
+        return launch_pdl(k_step<M>, dim3(pack_max(pk, m, [](const PatchDev& p) { return p.nblk_c; }), m), kTpb, 0, st,
+                          pk);
+    });
 }
 
-cudaError_t launch_compact(const PatchDev& p, cudaStream_t st) {
-    const cudaError_t e = launch_pdl(k_compact_scatter, p.nblk_c, kTpb, 0, st, p);
-    count_launches(1);
-    return e;
-}
-
-cudaError_t launch_inject(const PatchDev& p, const InjectParams& ip, cudaStream_t st) {
-    int blocks = (ip.total + kTpb - 1) / kTpb;
-    if (blocks < 1) blocks = 1;
-    if (blocks > 1024) blocks = 1024;
-    const cudaError_t e = launch_pdl(k_inject, blocks, kTpb, 0, st, p, ip);
-    count_launches(1);
-    return e;
-}
-
-cudaError_t launch_inject_dev(const PatchDev& p, const InjectParams* ip, cudaStream_t st) {
-    const cudaError_t e = launch_pdl(k_inject_dev, 152 * 2, kTpb, 0, st, p, ip);
-    count_launches(1);
-    return e;
-}
-
-cudaError_t launch_bin(const PatchDev& p, cudaStream_t st) {
-    // one block per key tile: keys, ids and every pass's digit totals
-    const int passes = (p.key_bits + 7) / 8;
-    // the sort passes: a persistent grid of the blocks that fit at once
-    const int per_sm = sort_pass_blocks_per_sm(), sms = sm_count();
-    const int grid = std::max(1, std::min(p.nblk_o, std::max(1, per_sm) * std::max(1, sms)));
-    cudaError_t e = launch_pdl(k_bin_keys, p.nblk_s, kTpb, 0, st, p, p.keys[0], p.vals[0], passes);
-    int src = 0;
-    for (int ps = 0; ps < passes && e == cudaSuccess; ++ps) {
-        e = launch_pdl(k_sort_pass, grid, kTpb, 0, st, (const uint32_t*)p.keys[src],
-                       (const uint32_t*)p.vals[src], p.keys[1 - src], p.vals[1 - src], (const int32_t*)p.count,
-                       8 * ps, p.hist + 256 * ps, p.sort_status + (size_t)ps * p.nblk_o * 256,
-                       p.sort_ticket + 2 * ps, p.stats + 2, kLbWaitCycles, 0);
-        src = 1 - src;
+cudaError_t launch_inject(const PatchDev* ps, const InjectParams* ips, int n, cudaStream_t st) {
+    auto blocks = [](int total) { return std::min(1024, std::max(1, (total + kTpb - 1) / kTpb)); };
+    // the patches that inject in this frame
+    int idx[kInjectMax];
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < n && e == cudaSuccess;) {
+        int m = 0, used = 0, most = 1;
+        for (; k < n && m < kInjectMax; ++k) {
+            const InjectParams& ip = ips[k];
+            if (ip.total <= 0) continue;
+            const int need = ip.nseg * (int)(sizeof(Segment) / 4) + 3 * ip.given;
+            if (m > 0 && used + need > kInjectWords) break;
+            idx[m++] = k;
+            used += need;
+            most = std::max(most, blocks(ip.total));
+        }
+        if (m == 0) break;
+        count_launches(1);
+        if (m == 1) {
+            e = launch_pdl(k_inject, most, kTpb, 0, st, ps[idx[0]], ips[idx[0]]);
+            continue;
+        }
+        InjectPack pk;
+        int w = 0;
+        for (int j = 0; j < m; ++j) {
+            const InjectParams& ip = ips[idx[j]];
+            pk.p[j] = ps[idx[j]];
+            pk.h[j] = InjectHead{ip.nseg, ip.total, ip.frame, ip.patch, ip.seed, ip.W, ip.H, ip.nth};
+            pk.seg0[j] = w;
+            memcpy(pk.words + w, ip.seg, ip.nseg * sizeof(Segment));
+            w += ip.nseg * (int)(sizeof(Segment) / 4);
+            pk.giv0[j] = w;
+            pk.given[j] = ip.given;
+            for (const int32_t* src : {ip.gx, ip.gy, ip.ga}) {
+                memcpy(pk.words + w, src, ip.given * sizeof(int32_t));
+                w += ip.given;
+            }
+        }
+        e = launch_pdl(k_inject_pack, dim3(most, m), kTpb, 0, st, pk);
     }
-    int rb = (2 * p.cap + 1 + kTpb * kRecItems - 1) / (kTpb * kRecItems);
-    rb = std::max(1, std::min(rb, std::max(1, sm_count()) * 8));
-    if (e == cudaSuccess)
-        e = launch_pdl(k_offsets_records, rb, kTpb, 0, st, p, (const uint32_t*)p.keys[src],
-                       (const uint32_t*)p.vals[src]);
-    count_launches(2 + passes);
     return e;
 }
 
-int sorted_buffer_index(const PatchDev& p) { return ((p.key_bits + 7) / 8) & 1; }
+cudaError_t launch_inject_dev(const PatchDev* ps, const InjectParams* ips_dev, int n, cudaStream_t st) {
+    const InjectParams* d = ips_dev;
+    return for_packs(ps, n, [&](const auto& pk, int m) {
+        constexpr int M = std::decay_t<decltype(pk)>::kM;
+        count_launches(1);
+        // the frame's counts are not known here: 8,192 particles a pass of the grid
+        const cudaError_t e = launch_pdl(k_inject_dev<M>, dim3(32, m), kTpb, 0, st, pk, d);
+        d += m;
+        return e;
+    });
+}
+
+cudaError_t launch_bin(const PatchDev* ps, int n, bool keys, cudaStream_t st) {
+    return for_packs(ps, n, [&](const auto& pk, int m) {
+        constexpr int M = std::decay_t<decltype(pk)>::kM;
+        const int passes = pack_max(pk, m, [](const PatchDev& p) { return sort_passes(p); });
+        cudaError_t e = keys ? launch_keys(pk, m, st) : cudaSuccess;
+        for (int s = 0; s < passes && e == cudaSuccess; ++s) e = launch_sort(pk, m, s, kLbWaitCycles, 0, st);
+        if (e != cudaSuccess) return e;
+        const int rb = pack_max(pk, m, [](const PatchDev& p) {
+            return (2 * (int64_t)p.cap + 1 + kTpb * kRecItems - 1) / (kTpb * kRecItems);
+        });
+        count_launches(1);
+        return launch_pdl(k_offsets_records<M>, dim3(std::min(rb, std::max(1, sm_count()) * 8), m), kTpb, 0, st, pk);
+    });
+}
+
+int sorted_buffer_index(const PatchDev& p) { return sort_passes(p) & 1; }
 
 cudaError_t launch_sort_stall(const PatchDev& p, long long wait_cycles, cudaStream_t st) {
     // the frame's keys and digit totals, then the first pass with tile 0
     // never taken: every block that looks back to it waits wait_cycles
-    const int passes = (p.key_bits + 7) / 8;
-    const int per_sm = sort_pass_blocks_per_sm(), sms = sm_count();
-    const int grid = std::max(1, std::min(p.nblk_o, std::max(1, per_sm) * std::max(1, sms)));
-    cudaError_t e = launch_pdl(k_bin_keys, p.nblk_s, kTpb, 0, st, p, p.keys[0], p.vals[0], passes);
-    if (e == cudaSuccess)
-        e = launch_pdl(k_sort_pass, grid, kTpb, 0, st, (const uint32_t*)p.keys[0], (const uint32_t*)p.vals[0],
-                       p.keys[1], p.vals[1], (const int32_t*)p.count, 0, p.hist, p.sort_status, p.sort_ticket,
-                       p.stats + 2, wait_cycles, 1);
-    count_launches(2);
-    return e;
+    PatchPack<1> pk;
+    pk.p[0] = p;
+    const cudaError_t e = launch_keys(pk, 1, st);
+    return e == cudaSuccess ? launch_sort(pk, 1, 0, wait_cycles, 1, st) : e;
 }
 
 }  // namespace scwp
