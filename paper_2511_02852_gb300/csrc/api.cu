@@ -970,7 +970,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
         ok = ok && P->d_items && P->d_spans && P->d_sat_items && P->d_sat_spans;
         const int G = P->partial_planes;
         if (G > 1) {
-            D.partial = (float*)dalloc(ctx, (size_t)G * 3 * T.W * T.H * sizeof(float));
+            D.partial = (float*)dalloc(ctx, (size_t)G * 3 * partial_pitch(T.W) * T.H * sizeof(float));
             ok = ok && D.partial;
         }
     }

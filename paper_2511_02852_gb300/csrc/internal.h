@@ -81,7 +81,7 @@ struct PatchDev {
                                           // kernel for the record pass's gathers
     BumpRec* rec = nullptr;               // [2 cap] bump records in bin order
     float* out = nullptr;                 // [3][H][W] blended maps
-    float* partial = nullptr;             // [groups][3][H][W] per-bucket-group sums (groups > 1)
+    float* partial = nullptr;             // [groups][3][H][partial_pitch(W)] per-bucket-group sums (groups > 1)
     int groups = 1;                       // bucket groups of the CUDA-core synthesis
     int groups_tc = 1;                    // bucket groups of the tensor-core synthesis
     int patch = 0;                        // index of the patch in its context
@@ -114,6 +114,12 @@ __host__ __device__ inline int item_groups(const TcItem& it) { return it.groups 
 __host__ __device__ inline int item_parts(const TcItem& it) { return (it.groups >> 16) > 1 ? (it.groups >> 16) : 1; }
 __host__ __device__ inline int item_group(const TcItem& it) { return it.group & 0xFFFF; }
 __host__ __device__ inline int item_part(const TcItem& it) { return it.group >> 16; }
+
+// Row pitch of the partial planes in texels: a multiple of four, so that the
+// blend reads (and a synthesis may write) whole aligned quads whatever the
+// patch's width.  Read by single texels (rows of odd widths are not aligned),
+// the blend of a 500-texel patch in 12 groups took 16 us.
+__host__ __device__ inline int partial_pitch(int W) { return (W + 3) & ~3; }
 
 // One span of the group-sum blend: quads [q0, q1) (4 texels of a row) of
 // patch `patch`, whose synthesis used `groups` bucket groups.
@@ -263,8 +269,8 @@ cudaError_t launch_normals(const float* maps, int W, int H, float cell, float* d
 // group sums and blend of `n_spans` spans of any patches, one launch
 cudaError_t launch_blend_spans(const BlendSpan* spans, int n_spans, const PatchDev* pdevs, const SynthParams* sps,
                                cudaStream_t st);
-// sum `groups` partial [3][H][W] planes at src (in order), blend, store to p.out
-cudaError_t launch_blend(const PatchDev& p, const SynthParams& sp, const float* src, int groups,
+// sum `groups` partial [3][H][pitch] planes at src (in order), blend, store to p.out
+cudaError_t launch_blend(const PatchDev& p, const SynthParams& sp, const float* src, int pitch, int groups,
                          cudaStream_t st);
 // layered variant: scratch (p.layers) must hold layered_scratch_bytes()
 size_t layered_scratch_bytes(const PatchDev& p, const int32_t* R_host);

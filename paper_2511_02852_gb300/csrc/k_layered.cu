@@ -197,7 +197,7 @@ cudaError_t launch_layered(const PatchDev& p, const SynthParams& sp, const int32
         launches += 3;
     }
     count_launches(launches);
-    return launch_blend(p, sp, acc, 1, st);
+    return launch_blend(p, sp, acc, p.W, 1, st);
 }
 
 }  // namespace scwp

@@ -189,11 +189,12 @@ __device__ __forceinline__ float blend_at(const SynthParams& sp, int ix, int iy,
     return w;
 }
 
-// store 4 consecutive texels of row iy for the three fields
-__device__ __forceinline__ void store_row4(float* out, size_t plane, int W, int iy, int ix0,
+// store 4 consecutive texels of row iy for the three fields (rows of `pitch`
+// texels, W of them in use)
+__device__ __forceinline__ void store_row4(float* out, size_t plane, int W, int pitch, int iy, int ix0,
                                            const float o[3][4]) {
-    const size_t rowo = (size_t)iy * W;
-    if ((W & 3) == 0 && ix0 + 3 < W) {
+    const size_t rowo = (size_t)iy * pitch;
+    if ((pitch & 3) == 0 && ix0 + 3 < pitch) {
 #pragma unroll
         for (int f = 0; f < 3; ++f)
             *reinterpret_cast<float4*>(out + f * plane + rowo + ix0) =
@@ -208,62 +209,70 @@ __device__ __forceinline__ void store_row4(float* out, size_t plane, int W, int 
 }
 
 // sum of the bucket-group partials (in group order) and the blend of quad q
-// (texels 4 (q mod qw) .. + 3 of row q / qw)
-__device__ __forceinline__ void blend_quad(const PatchDev& p, const SynthParams& sp, const float* partial,
+// (texels 4 (q mod qw) .. + 3 of row q / qw).  The background samples come
+// first and the groups' loads four at a time, so that a thread's loads are
+// in flight together: with a few hundred CTAs at most the pass is bound by
+// latency, not by the planes' bytes.
+__device__ __forceinline__ void blend_quad(float* out, const SynthParams& sp, const float* partial, int pitch,
                                            int groups, int q) {
-    const size_t plane = (size_t)sp.W * sp.H;
+    const size_t plane = (size_t)sp.W * sp.H, src_plane = (size_t)pitch * sp.H;
     const int qw = (sp.W + 3) / 4;
     const int iy = q / qw, ix0 = 4 * (q - iy * qw);
-    float acc[3][4];
+    float w[4], bgv[4][3], acc[3][4];
+#pragma unroll
+    for (int cc = 0; cc < 4; ++cc) w[cc] = blend_at(sp, ix0 + cc, iy, bgv[cc]);
 #pragma unroll
     for (int f = 0; f < 3; ++f)
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) acc[f][cc] = 0.f;
-    const size_t rowo = (size_t)iy * sp.W;
-    const bool vec = (sp.W & 3) == 0 && ix0 + 3 < sp.W;
-    for (int g = 0; g < groups; ++g) {
-        const float* src = partial + (size_t)g * 3 * plane;
+    const float* src = partial + (size_t)iy * pitch + ix0;
+    if ((pitch & 3) == 0) {   // (uniform) then ix0 + 3 < pitch
+#pragma unroll 4
+        for (int g = 0; g < groups; ++g) {
 #pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            if (vec) {
-                const float4 v = *reinterpret_cast<const float4*>(src + f * plane + rowo + ix0);
+            for (int f = 0; f < 3; ++f) {
+                const float4 v = *reinterpret_cast<const float4*>(src + ((size_t)g * 3 + f) * src_plane);
                 acc[f][0] += v.x;
                 acc[f][1] += v.y;
                 acc[f][2] += v.z;
                 acc[f][3] += v.w;
-            } else {
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc)
-                    if (ix0 + cc < sp.W) acc[f][cc] += src[f * plane + rowo + ix0 + cc];
             }
         }
+    } else {
+        for (int g = 0; g < groups; ++g)
+#pragma unroll
+            for (int f = 0; f < 3; ++f)
+#pragma unroll
+                for (int cc = 0; cc < 4; ++cc)
+                    if (ix0 + cc < sp.W) acc[f][cc] += src[((size_t)g * 3 + f) * src_plane + cc];
     }
     float o[3][4];
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-        float bgv[3];
-        const float w = blend_at(sp, ix0 + cc, iy, bgv);
+    for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
-        for (int f = 0; f < 3; ++f) o[f][cc] = w * acc[f][cc] + (1.f - w) * bgv[f];
-    }
-    store_row4(p.out, plane, sp.W, iy, ix0, o);
+        for (int f = 0; f < 3; ++f) o[f][cc] = w[cc] * acc[f][cc] + (1.f - w[cc]) * bgv[cc][f];
+    store_row4(out, plane, sp.W, sp.W, iy, ix0, o);
 }
 
-__global__ void __launch_bounds__(256) k_blend_groups(PatchDev p, SynthParams sp, const float* partial,
+__global__ void __launch_bounds__(256) k_blend_groups(PatchDev p, SynthParams sp, const float* partial, int pitch,
                                                       int groups) {
     const int nq = ((sp.W + 3) / 4) * sp.H;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x)
-        blend_quad(p, sp, partial, groups, q);
+        blend_quad(p.out, sp, partial, pitch, groups, q);
 }
 
-// the same over spans of any patches: one CTA per span
+// the same over spans of any patches: one CTA per span.  The span and the
+// patch's descriptors are read before the synthesis ahead of this launch is
+// done: they were written before that synthesis started.
 __global__ void __launch_bounds__(256) k_blend_spans(const BlendSpan* spans, const PatchDev* pdevs,
                                                      const SynthParams* sps) {
-    pdl_enter();
     const BlendSpan sn = spans[blockIdx.x];
-    const PatchDev& p = pdevs[sn.patch];
-    const SynthParams& sp = sps[sn.patch];
-    for (int q = sn.q0 + threadIdx.x; q < sn.q1; q += blockDim.x) blend_quad(p, sp, p.partial, sn.groups, q);
+    float* const out = pdevs[sn.patch].out;
+    const float* const partial = pdevs[sn.patch].partial;
+    const SynthParams sp = sps[sn.patch];
+    pdl_enter();
+    for (int q = sn.q0 + threadIdx.x; q < sn.q1; q += blockDim.x)
+        blend_quad(out, sp, partial, partial_pitch(sp.W), sn.groups, q);
 }
 
 __global__ void __launch_bounds__(kThreads, 2) k_synth_gather(PatchDev p, SynthParams sp) {
@@ -478,7 +487,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_synth_gather(PatchDev p, SynthP
     if (G > 1) {
         // raw sums of this bucket group; k_blend_groups adds the groups in
         // order and blends
-        float* dst = p.partial + (size_t)g * 3 * plane;
+        const int pitch = partial_pitch(sp.W);
+        const size_t pplane = (size_t)pitch * sp.H;
+        float* dst = p.partial + (size_t)g * 3 * pplane;
 #pragma unroll
         for (int r = 0; r < kRPT; ++r) {
             const int iy = ty0 + kRPT * tr + r;
@@ -486,7 +497,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_synth_gather(PatchDev p, SynthP
             const float o[3][4] = {{h[r][0], h[r][1], h[r][2], h[r][3]},
                                    {dx[r][0], dx[r][1], dx[r][2], dx[r][3]},
                                    {dy[r][0], dy[r][1], dy[r][2], dy[r][3]}};
-            store_row4(dst, plane, sp.W, iy, tx0 + kCPT * tc, o);
+            store_row4(dst, pplane, sp.W, pitch, iy, tx0 + kCPT * tc, o);
         }
         return;
     }
@@ -504,7 +515,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_synth_gather(PatchDev p, SynthP
             o[1][cc] = w * dx[r][cc] + (1.f - w) * bgv[1];
             o[2][cc] = w * dy[r][cc] + (1.f - w) * bgv[2];
         }
-        store_row4(p.out, plane, sp.W, iy, tx0 + kCPT * tc, o);
+        store_row4(p.out, plane, sp.W, sp.W, iy, tx0 + kCPT * tc, o);
     }
 }
 
@@ -518,7 +529,7 @@ cudaError_t launch_synth_gather(const PatchDev& p, const SynthParams& sp, cudaSt
     dim3 grid((p.W + kTX - 1) / kTX, (p.H + kTY - 1) / kTY, G);
     k_synth_gather<<<grid, kThreads, sm, st>>>(p, sp);
     count_launches(1);
-    if (G > 1) return launch_blend(p, sp, p.partial, G, st);
+    if (G > 1) return launch_blend(p, sp, p.partial, partial_pitch(sp.W), G, st);
     return cudaGetLastError();
 }
 
@@ -529,12 +540,12 @@ cudaError_t launch_blend_spans(const BlendSpan* spans, int n_spans, const PatchD
     return e;
 }
 
-cudaError_t launch_blend(const PatchDev& p, const SynthParams& sp, const float* src, int groups,
+cudaError_t launch_blend(const PatchDev& p, const SynthParams& sp, const float* src, int pitch, int groups,
                          cudaStream_t st) {
     const int nq = ((p.W + 3) / 4) * p.H;
     int blocks = (nq + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    k_blend_groups<<<blocks, 256, 0, st>>>(p, sp, src, groups);
+    k_blend_groups<<<blocks, 256, 0, st>>>(p, sp, src, pitch, groups);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -524,7 +524,8 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
         // ---- store: the item's partial plane, or (one plane) the blended maps
         const int x = tx0 + cx;
         if (x < sp.W) {
-            const size_t plane = (size_t)sp.W * sp.H;
+            const int pitch = G * K > 1 ? partial_pitch(sp.W) : sp.W;
+            const size_t plane = (size_t)pitch * sp.H;
             const int pl = g * K + part;
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
@@ -534,7 +535,7 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 for (int r = 0; r < kSegRows; ++r) {
                     const int y = ty0 + sg * kSegRows + r;
                     const float v = f == 0 ? ah[r] : (f == 1 ? adx[r] : ady[r]);
-                    if (y < sp.H) dst[(size_t)y * sp.W] = G * K > 1 ? v : blend1(sp, x, y, f, v);
+                    if (y < sp.H) dst[(size_t)y * pitch] = G * K > 1 ? v : blend1(sp, x, y, f, v);
                 }
             }
         }

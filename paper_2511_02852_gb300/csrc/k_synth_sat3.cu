@@ -361,7 +361,8 @@ __global__ void __launch_bounds__(kSatThreads, 2) k_synth_sat3(const TcItem* ite
     // ---- store: the group's partial planes, or (one group) the blended maps
     const int x = tx0 + cx;
     if (x >= sp.W) return;
-    const size_t plane = (size_t)sp.W * sp.H;
+    const int pitch = G * K > 1 ? partial_pitch(sp.W) : sp.W;
+    const size_t plane = (size_t)pitch * sp.H;
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
         float* const dst =
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(kSatThreads, 2) k_synth_sat3(const TcItem* ite
         for (int r = 0; r < kSegRows; ++r) {
             const int y = ty0 + sg * kSegRows + r;
             const float v = f == 0 ? ah[r] : (f == 1 ? adx[r] : ady[r]);
-            if (y < sp.H) dst[(size_t)y * sp.W] = G * K > 1 ? v : blend1(sp, x, y, f, v);
+            if (y < sp.H) dst[(size_t)y * pitch] = G * K > 1 ? v : blend1(sp, x, y, f, v);
         }
     }
 }

@@ -691,11 +691,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_synth_tc(const TcItem* items, c
             const int Wd = sp.W, Hd = sp.H;
             if (x >= Wd) continue;
             // bucket groups: this group's partial plane; one group: the blended map
-            float* const dst = (G > 1 ? p.partial + ((size_t)g * 3 + f) * plane : p.out + (size_t)f * plane) + x;
+            const int pitch = G > 1 ? partial_pitch(Wd) : Wd;
+            float* const dst =
+                (G > 1 ? p.partial + ((size_t)g * 3 + f) * pitch * Hd : p.out + (size_t)f * plane) + x;
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 const int y = y0 + j;
-                if (y < Hd) dst[(size_t)y * Wd] = G > 1 ? val[j] : blend1(sp, x, y, f, val[j]);
+                if (y < Hd) dst[(size_t)y * pitch] = G > 1 ? val[j] : blend1(sp, x, y, f, val[j]);
             }
         }
     }
