@@ -39,9 +39,14 @@
 // heaviest-first order; the last CTA to finish resets the queue for the next
 // launch, so no CTA ever waits on another).  All nine S_ij planes of a
 // bucket live in shared memory at once (144 KB), so each candidate bump
-// enters exactly once per pass.  Per item, the buckets' bin geometry and the
-// bin rows that reach the tile are read once into a row table (a bucket with
-// more rows than the table spans several segments, each a pass of its own).
+// enters exactly once per pass.  An item is worked off in batches: the bin
+// rows of its buckets that reach the tile are read into a row table (all of
+// them, in nearly every item; a bucket with more rows than the table spans
+// several segments, each a pass of its own).  Two batches are held: eight
+// warps build the next one (the next item's ticket, descriptors, bucket
+// geometry and row table: five dependent round trips to L2) in the y-prefix
+// phase of this one's last pass but one, which leaves them idle, so an item
+// starts without a wait and its first records are already on their way.
 // Within a pass each thread takes the candidates c0 + tid, c0 + tid + 1024,
 // ... on its own, with no barrier until the pass ends: it finds a
 // candidate's bin row (a binary search of the row table) and copies the
@@ -80,24 +85,37 @@ constexpr int kRowCap = 256;                 // bin rows held at once (all segme
 constexpr int kMaxSeg = 64;                  // segments per batch
 constexpr int32_t kQs = 65536, kHalfs = 32768;
 static_assert(kSegs * kSegRows == kT && kSegs == 16, "contraction mapping");
-static_assert(kScanThreads % 32 == 0 && kScanThreads + 128 <= kSatThreads, "scan warps and helper warps");
+static_assert(kScanThreads % 32 == 0, "whole scan warps");
+
+constexpr int kBuildWarp0 = 24;              // warps 24 .. 31 build the next batch
+constexpr int kBuildThreads = kSatThreads - 32 * kBuildWarp0;
+static_assert(kScanThreads + 2 * kT <= 32 * kBuildWarp0, "phase threads and builders apart");
+
+// A batch of one item: segments (bucket, row range) whose bin rows fit the row table.
+struct Batch {
+    int32_t rs[kRowCap];                  // first record of each bin row of the batch
+    int32_t cum[kRowCap];                 // candidates of the segment before the row
+    // the segments: bucket, half-width, |A| bound, first table row, candidates, candidates per pass
+    int32_t sgb[kMaxSeg], sgR[kMaxSeg], sgrb[kMaxSeg + 1], sgnc[kMaxSeg], sgm[kMaxSeg];
+    float sgA[kMaxSeg];
+    int32_t item, nseg, last;             // last: the item's last batch
+    int32_t t_next, r0_next;              // else the bucket (item-relative) and row the next one starts at
+    int32_t tx0, ty0, planes, plane, K, part;   // partial planes of the item's tile and its own; parts
+    int32_t patch;                        // the patch whose descriptors pd, spd hold (-1: none)
+    alignas(16) unsigned char pd[sizeof(PatchDev)];
+    alignas(16) unsigned char spd[sizeof(SynthParams)];
+};
 
 struct SatSmem {
     uint32_t E[kPlanes][kT * kT];         // difference arrays, then prefix sums; zero between passes
     alignas(128) BumpRec raw[2][kSatThreads];   // two record slots per thread
-    float2 ph[2][2 * kT];                 // texel phases (cos, sin) a of a segment's bucket: rows, then columns
-    int32_t rs[kRowCap];                  // first record of each bin row of the batch
-    int32_t cum[kRowCap];                 // candidates of the segment before the row
-    // the item's buckets
-    int32_t mR[kMaxBuckets], mC[kMaxBuckets], mnbx[kMaxBuckets], mbase[kMaxBuckets];
+    alignas(16) float2 ph[2 * kT];        // texel phases (cos, sin) a of the pass's bucket: rows, then columns
+    Batch bt[2];
+    // the builders' table of the item's buckets, and the segments' first rows
+    int32_t mR[kMaxBuckets], mnbx[kMaxBuckets], mbase[kMaxBuckets];
     int32_t mbx_lo[kMaxBuckets], mbx_hi[kMaxBuckets], mby_lo[kMaxBuckets], mnrows[kMaxBuckets];
     float mamax[kMaxBuckets], msatc[kMaxBuckets];
-    // the batch's segments: bucket (item-relative), first row, first table
-    // row, candidates, candidates per pass
-    int32_t sgb[kMaxSeg], sgr0[kMaxSeg], sgrb[kMaxSeg + 1], sgnc[kMaxSeg], sgm[kMaxSeg];
-    int32_t item, patch, nseg, bt_next, bt_r0, pad;
-    alignas(16) unsigned char pd[sizeof(PatchDev)];
-    alignas(16) unsigned char spd[sizeof(SynthParams)];
+    int32_t sgr0[kMaxSeg];
 };
 static_assert(sizeof(SatSmem) <= 227 * 1024, "shared memory of one CTA");
 static_assert(sizeof(BumpRec) == 32, "32-byte records (two 16-byte copies)");
@@ -158,44 +176,206 @@ struct Pass {
     int s, c0, c1;
 };
 
-__device__ __forceinline__ Pass make_pass(const SatSmem& S, int s, int c0) {
-    return Pass{s, c0, min(S.sgnc[s], c0 + S.sgm[s])};
+__device__ __forceinline__ Pass make_pass(const Batch& B, int s, int c0) {
+    return Pass{s, c0, min(B.sgnc[s], c0 + B.sgm[s])};
 }
 
 // The part's first pass of segments s0, s0 + 1, ... with candidates.
-__device__ __forceinline__ Pass first_pass_from(const SatSmem& S, int s0, int nseg, int part) {
-    for (int s = s0; s < nseg; ++s)
-        if (part * S.sgm[s] < S.sgnc[s]) return make_pass(S, s, part * S.sgm[s]);
+__device__ __forceinline__ Pass first_pass_from(const Batch& B, int s0) {
+    for (int s = s0; s < B.nseg; ++s)
+        if (B.part * B.sgm[s] < B.sgnc[s]) return make_pass(B, s, B.part * B.sgm[s]);
     return Pass{-1, 0, 0};
 }
 
 // The pass after P in this part's order: the part's next pass of the same
 // segment (parts take every K-th pass), else the first of a later segment.
-__device__ __forceinline__ Pass next_pass(const SatSmem& S, Pass P, int nseg, int K, int part) {
-    const int c0 = P.c0 + K * S.sgm[P.s];
-    if (c0 < S.sgnc[P.s]) return make_pass(S, P.s, c0);
-    return first_pass_from(S, P.s + 1, nseg, part);
+__device__ __forceinline__ Pass next_pass(const Batch& B, Pass P) {
+    const int c0 = P.c0 + B.K * B.sgm[P.s];
+    if (c0 < B.sgnc[P.s]) return make_pass(B, P.s, c0);
+    return first_pass_from(B, P.s + 1);
 }
 
 // This thread's copy of candidate j (of the segment whose table rows are
-// [lo, hi]) into its slot `slot`; returns the candidate's row.  The row is
-// the last one that starts at or before j (empty rows start where the next
-// one does).
-__device__ __forceinline__ int fetch_rows(SatSmem& S, const BumpRec* rec, int lo, int hi, int j, int slot, int tid) {
-    if (lo < hi && S.cum[lo + 1] > j) hi = lo;   // still the row of the hint
+// [lo, hi]) into its slot; returns the candidate's row.  The row is the last
+// one that starts at or before j (empty rows start where the next one does).
+__device__ __forceinline__ int fetch_rows(BumpRec* slot, const Batch& B, int lo, int hi, int j, int tid) {
+    if (lo < hi && B.cum[lo + 1] > j) hi = lo;   // still the row of the hint
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (S.cum[mid] <= j)
+        if (B.cum[mid] <= j)
             lo = mid;
         else
             hi = mid - 1;
     }
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(rec + S.rs[lo] + (j - S.cum[lo]));
-    unsigned char* dst = reinterpret_cast<unsigned char*>(&S.raw[slot][tid]);
+    const BumpRec* const rec = reinterpret_cast<const PatchDev*>(B.pd)->rec;
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(rec + B.rs[lo] + (j - B.cum[lo]));
+    unsigned char* dst = reinterpret_cast<unsigned char*>(slot + tid);
     const int hs = half_swap(tid);
     cp_async16(dst + 16 * hs, src);
     cp_async16(dst + 16 * (hs ^ 1), src + 16);
     return lo;
+}
+
+// ... of this thread's first candidate of pass P, if it has one
+__device__ __forceinline__ void fetch_first(BumpRec* slot, const Batch& B, Pass P, int tid) {
+    if (P.s >= 0 && P.c0 + tid < P.c1)
+        fetch_rows(slot, B, B.sgrb[P.s], B.sgrb[P.s + 1] - 1, P.c0 + tid, tid);
+}
+
+__device__ __forceinline__ void builders_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(kBuildThreads) : "memory");
+}
+
+// Build the batch after batch nx ^ 1 into batch nx (the eight builder warps;
+// bt: thread among them): more of the same item if that one was not its
+// last, else the next item of the queue.  Readers need a block barrier.
+__device__ void build_batch(SatSmem& S, int nx, bool more, const TcItem* items, int n_items, const PatchDev* pdevs,
+                            const SynthParams* sps, unsigned int* queue, int bt) {
+    Batch& B = S.bt[nx];
+    const Batch& A = S.bt[nx ^ 1];
+    const int lane = bt & 31, bw = bt >> 5;
+    if (bt == 0) B.item = more ? A.item : (int)atomicAdd(queue, 1u);
+    builders_sync();
+    const int ti = B.item;
+    if (ti >= n_items) return;
+    const TcItem it = items[ti];
+    if (it.patch != B.patch) {   // (uniform) items of one patch share its descriptors
+        static_assert(sizeof(PatchDev) % 4 == 0 && sizeof(SynthParams) % 4 == 0, "descriptor copy");
+        const uint32_t* a = reinterpret_cast<const uint32_t*>(pdevs + it.patch);
+        const uint32_t* b = reinterpret_cast<const uint32_t*>(sps + it.patch);
+        for (int k = bt; k < (int)(sizeof(PatchDev) / 4); k += kBuildThreads) reinterpret_cast<uint32_t*>(B.pd)[k] = a[k];
+        for (int k = bt; k < (int)(sizeof(SynthParams) / 4); k += kBuildThreads)
+            reinterpret_cast<uint32_t*>(B.spd)[k] = b[k];
+        builders_sync();
+        if (bt == 0) B.patch = it.patch;
+    }
+    const PatchDev& p = *reinterpret_cast<const PatchDev*>(B.pd);
+    const SynthParams& sp = *reinterpret_cast<const SynthParams*>(B.spd);
+    const int G = item_groups(it), g = item_group(it), K = item_parts(it), part = item_part(it);
+    const int ntx = (sp.W + kT - 1) / kT;
+    const int tx0 = (it.tile % ntx) * kT, ty0 = (it.tile / ntx) * kT;
+    const int b_begin = max((g * sp.nb) / G, sp.b_lo);
+    const int nbk = max(0, min(((g + 1) * sp.nb) / G, sp.b_hi) - b_begin);
+    // Q16.16 centres of the tile's first and last texel columns and rows
+    const int32_t X0 = tx0 * kQs + kHalfs, X1 = X0 + (kT - 1) * kQs;
+    const int32_t Y0 = ty0 * kQs + kHalfs, Y1 = Y0 + (kT - 1) * kQs;
+    // ---- the item's buckets, one thread each: bins hold x_b + R in
+    // [bx C, (bx + 1) C); the bin rows and columns that reach the tile
+    static_assert(kMaxBuckets <= 64 && kMaxSeg >= kMaxBuckets && kMaxBuckets <= kBuildThreads, "two buckets per lane");
+    if (bt < nbk) {
+        const BucketDev bk = p.bk[b_begin + bt];
+        const float amax = p.amax[b_begin + bt];
+        const int bx_lo = (int)((int64_t)X0 / bk.C);
+        const int bx_hi = min((int)(((int64_t)X1 + 2 * (int64_t)bk.R - 1) / bk.C), bk.nbx - 1);
+        const int by_lo = (int)((int64_t)Y0 / bk.C);
+        const int by_hi = min((int)(((int64_t)Y1 + 2 * (int64_t)bk.R - 1) / bk.C), bk.nby - 1);
+        S.mR[bt] = bk.R;
+        S.mnbx[bt] = bk.nbx;
+        S.mbase[bt] = bk.base;
+        S.mbx_lo[bt] = bx_lo;
+        S.mbx_hi[bt] = bx_hi;
+        S.mby_lo[bt] = by_lo;
+        S.mnrows[bt] = (bx_lo > bx_hi || by_lo > by_hi || !(amax > 0.f)) ? 0 : by_hi - by_lo + 1;
+        S.mamax[bt] = amax;
+        S.msatc[bt] = bk.sat_c;
+    }
+    builders_sync();
+    // ---- segments (bucket, row range) whose bin rows fit the row table
+    if (bw == 0) {
+        const int t0 = more ? A.t_next : 0, r0 = more ? A.r0_next : 0;
+        int rows[2], before[2], nrow = 0, n = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int t = lane + 32 * h;
+            rows[h] = t >= t0 && t < nbk ? S.mnrows[t] - (t == t0 ? r0 : 0) : 0;
+            const uint32_t inc = warp_scan((uint32_t)rows[h], lane);
+            before[h] = nrow + (int)inc - rows[h];
+            nrow += (int)__shfl_sync(0xffffffffu, inc, 31);
+        }
+        if (nrow <= kRowCap) {   // all that are left
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int t = lane + 32 * h;
+                const unsigned m = __ballot_sync(0xffffffffu, rows[h] > 0);
+                if (rows[h] > 0) {
+                    const int s = n + __popc(m & ((1u << lane) - 1u));
+                    B.sgb[s] = t;
+                    S.sgr0[s] = t == t0 ? r0 : 0;
+                    B.sgrb[s] = before[h];
+                }
+                n += __popc(m);
+            }
+            if (lane == 0) {
+                B.sgrb[n] = nrow;
+                B.nseg = n;
+                B.last = 1;
+            }
+        } else if (lane == 0) {
+            int rws = 0, t = t0, r = r0;
+            while (t < nbk && n < kMaxSeg) {
+                const int left = S.mnrows[t] - r;
+                if (left <= 0) {
+                    ++t;
+                    r = 0;
+                    continue;
+                }
+                const int take = min(left, kRowCap - rws);
+                if (take <= 0) break;
+                B.sgb[n] = t;
+                S.sgr0[n] = r;
+                B.sgrb[n] = rws;
+                rws += take;
+                ++n;
+                r += take;
+                if (r >= S.mnrows[t]) {
+                    ++t;
+                    r = 0;
+                }
+            }
+            B.sgrb[n] = rws;
+            B.nseg = n;
+            B.last = t >= nbk ? 1 : 0;
+            B.t_next = t;
+            B.r0_next = r;
+        }
+        if (lane == 0) {
+            B.tx0 = tx0;
+            B.ty0 = ty0;
+            B.planes = G * K;
+            B.plane = g * K + part;
+            B.K = K;
+            B.part = part;
+        }
+    }
+    builders_sync();
+    // ---- the row table: first record of every row, and the exclusive prefix
+    // of the rows' lengths within each segment (warp w: segments w, w + 8, ...)
+    for (int s = bw; s < B.nseg; s += kBuildThreads / 32) {
+        const int t = B.sgb[s], q0 = B.sgrb[s], q1 = B.sgrb[s + 1], nbx = S.mnbx[t];
+        const uint32_t* const off = p.offsets + (S.mbase[t] + (S.mby_lo[t] + S.sgr0[s]) * nbx);
+        const int lo = S.mbx_lo[t], hi = S.mbx_hi[t] + 1;
+        uint32_t carry = 0u;
+        for (int q = q0; q < q1; q += 32) {
+            uint32_t l = 0u;
+            if (q + lane < q1) {
+                const int r = (q - q0 + lane) * nbx;
+                const uint32_t s0 = off[r + lo];
+                l = off[r + hi] - s0;
+                B.rs[q + lane] = (int32_t)s0;
+            }
+            const uint32_t inc = warp_scan(l, lane);
+            if (q + lane < q1) B.cum[q + lane] = (int32_t)(carry + inc - l);
+            carry += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        if (lane == 0) {
+            B.sgnc[s] = (int32_t)carry;
+            B.sgm[s] = carry ? pass_size((int)carry, S.msatc[t]) : 0;
+            B.sgR[s] = S.mR[t];
+            B.sgA[s] = S.mamax[t];
+        }
+        __syncwarp();
+        if (lane == 0) B.sgb[s] = b_begin + t;   // (absolute from here on; only this warp reads it above)
+    }
 }
 
 // The record of this thread's slot (its two 16-byte halves in the order
@@ -225,171 +405,69 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
     // contraction: this thread owns texel column cx of rows sg*4 .. sg*4 + 3
     const int cx = tid & (kT - 1), sg = tid / kT;
     pdl_enter();
-    // E starts zeroed, and every pass leaves it zeroed again
-    {
+    if (warp >= kBuildWarp0) {   // the first item
+        const int bt = tid - 32 * kBuildWarp0;
+        if (bt < 2) S.bt[bt].patch = -1;
+        build_batch(S, 0, false, items, n_items, pdevs, sps, queue, bt);
+    } else {   // E starts zeroed, and every pass leaves it zeroed again
         uint4* e4 = reinterpret_cast<uint4*>(&S.E[0][0]);
-        for (int k = tid; k < kPlanes * kT * kT / 4; k += kSatThreads) e4[k] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    if (tid == 0) {
-        S.item = (int)atomicAdd(queue, 1u);
-        S.patch = -1;
+        for (int k = tid; k < kPlanes * kT * kT / 4; k += 32 * kBuildWarp0) e4[k] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
-    for (;;) {
-        const int ti = S.item;
-        if (ti >= n_items) break;
-        const TcItem it = items[ti];
-        if (it.patch != S.patch) {   // (uniform) items of one patch share its descriptors
-            static_assert(sizeof(PatchDev) % 4 == 0 && sizeof(SynthParams) % 4 == 0, "descriptor copy");
-            const uint32_t* a = reinterpret_cast<const uint32_t*>(pdevs + it.patch);
-            const uint32_t* b = reinterpret_cast<const uint32_t*>(sps + it.patch);
-            for (int k = tid; k < (int)(sizeof(PatchDev) / 4); k += kSatThreads)
-                reinterpret_cast<uint32_t*>(S.pd)[k] = a[k];
-            for (int k = tid; k < (int)(sizeof(SynthParams) / 4); k += kSatThreads)
-                reinterpret_cast<uint32_t*>(S.spd)[k] = b[k];
-            __syncthreads();
-            if (tid == 0) S.patch = it.patch;
-        }
-        const PatchDev& p = *reinterpret_cast<const PatchDev*>(S.pd);
-        const SynthParams& sp = *reinterpret_cast<const SynthParams*>(S.spd);
-        const int G = item_groups(it), g = item_group(it), K = item_parts(it), part = item_part(it);
-        const int ntx = (sp.W + kT - 1) / kT;
-        const int tx0 = (it.tile % ntx) * kT, ty0 = (it.tile / ntx) * kT;
-        const int b_begin = max((g * sp.nb) / G, sp.b_lo);
-        const int b_end = min(((g + 1) * sp.nb) / G, sp.b_hi);
-        const int nbk = max(0, b_end - b_begin);
-        // Q16.16 centres of the tile's first and last texel columns and rows
-        const int32_t X0 = tx0 * kQs + kHalfs, X1 = X0 + (kT - 1) * kQs;
-        const int32_t Y0 = ty0 * kQs + kHalfs, Y1 = Y0 + (kT - 1) * kQs;
-        const float lamq = 0.5f * sp.lam_half;   // lam / 4
-        // ---- the item's buckets, one thread each: bins hold x_b + R in
-        // [bx C, (bx + 1) C); the bin rows and columns that reach the tile
-        for (int t = tid; t < nbk; t += kSatThreads) {
-            const BucketDev bk = p.bk[b_begin + t];
-            const float amax = p.amax[b_begin + t];
-            const int bx_lo = (int)((int64_t)X0 / bk.C);
-            const int bx_hi = min((int)(((int64_t)X1 + 2 * (int64_t)bk.R - 1) / bk.C), bk.nbx - 1);
-            const int by_lo = (int)((int64_t)Y0 / bk.C);
-            const int by_hi = min((int)(((int64_t)Y1 + 2 * (int64_t)bk.R - 1) / bk.C), bk.nby - 1);
-            S.mR[t] = bk.R;
-            S.mC[t] = bk.C;
-            S.mnbx[t] = bk.nbx;
-            S.mbase[t] = bk.base;
-            S.mbx_lo[t] = bx_lo;
-            S.mbx_hi[t] = bx_hi;
-            S.mby_lo[t] = by_lo;
-            S.mnrows[t] = (bx_lo > bx_hi || by_lo > by_hi || !(amax > 0.f)) ? 0 : by_hi - by_lo + 1;
-            S.mamax[t] = amax;
-            S.msatc[t] = bk.sat_c;
-        }
-        float ah[kSegRows], adx[kSegRows], ady[kSegRows];
+    float ah[kSegRows], adx[kSegRows], ady[kSegRows];
 #pragma unroll
-        for (int r = 0; r < kSegRows; ++r) ah[r] = adx[r] = ady[r] = 0.f;
-        int t_next = 0, sub_r0 = 0;   // the first bucket (and its row) not yet batched
-        for (;;) {
-            __syncthreads();   // bucket table written; the previous batch is done with the row table
-            // ---- a batch: segments (bucket, row range) whose bin rows fit the row table
-            // (a bucket with more rows than the table spans several segments)
-            if (tid == 0) {
-                int n = 0, rows = 0, t = t_next, r0 = sub_r0;
-                while (t < nbk && n < kMaxSeg) {
-                    const int left = S.mnrows[t] - r0;
-                    if (left <= 0) {
-                        ++t;
-                        r0 = 0;
-                        continue;
-                    }
-                    const int take = min(left, kRowCap - rows);
-                    if (take <= 0) break;
-                    S.sgb[n] = t;
-                    S.sgr0[n] = r0;
-                    S.sgrb[n] = rows;
-                    rows += take;
-                    ++n;
-                    r0 += take;
-                    if (r0 >= S.mnrows[t]) {
-                        ++t;
-                        r0 = 0;
-                    }
-                }
-                S.sgrb[n] = rows;
-                S.nseg = n;
-                S.bt_next = t;
-                S.bt_r0 = r0;
-            }
-            __syncthreads();
-            const int nseg = S.nseg;
-            t_next = S.bt_next;
-            sub_r0 = S.bt_r0;
-            if (nseg == 0) break;
-            // ---- the batch's row table: first record and length of every row
-            const int nq = S.sgrb[nseg];
-            for (int q = tid; q < nq; q += kSatThreads) {
-                int s = 0;
-                while (S.sgrb[s + 1] <= q) ++s;
-                const int t = S.sgb[s];
-                const int r = S.sgr0[s] + (q - S.sgrb[s]);
-                const int key0 = S.mbase[t] + (S.mby_lo[t] + r) * S.mnbx[t];
-                const int s0 = (int)p.offsets[key0 + S.mbx_lo[t]];
-                S.rs[q] = s0;
-                S.cum[q] = (int)p.offsets[key0 + S.mbx_hi[t] + 1] - s0;   // row length for now
-            }
-            __syncthreads();
-            // exclusive prefix of the row lengths within each segment (warp w:
-            // segments w, w + 32)
-            for (int s = warp; s < nseg; s += kSatThreads / 32) {
-                const int q0 = S.sgrb[s], q1 = S.sgrb[s + 1];
-                uint32_t carry = 0u;
-                for (int q = q0; q < q1; q += 32) {
-                    const uint32_t l = q + lane < q1 ? (uint32_t)S.cum[q + lane] : 0u;
-                    const uint32_t inc = warp_scan(l, lane);
-                    if (q + lane < q1) S.cum[q + lane] = (int32_t)(carry + inc - l);
-                    carry += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                if (lane == 0) {
-                    S.sgnc[s] = (int32_t)carry;
-                    S.sgm[s] = carry ? pass_size((int)carry, S.msatc[S.sgb[s]]) : 0;
-                }
-            }
-            __syncthreads();
-
-            // ---- the batch's passes of this part.  Invariant at a pass's
-            // start: if this thread has a candidate in it (c0 + tid < c1),
-            // its record is on the way into slot k (the last commit group).
-            Pass P = first_pass_from(S, 0, nseg, part);
-            int k = 0;
-            if (P.s >= 0 && P.c0 + tid < P.c1) fetch_rows(S, p.rec, S.sgrb[P.s], S.sgrb[P.s + 1] - 1, P.c0 + tid, k, tid);
+    for (int r = 0; r < kSegRows; ++r) ah[r] = adx[r] = ady[r] = 0.f;
+    int cur = 0, k = 0;         // the batch; the record slot of the next candidate
+    bool fetched = false;       // the batch's first copies are on their way
+    while (S.bt[cur].item < n_items) {
+        const Batch& B = S.bt[cur];
+        const PatchDev& p = *reinterpret_cast<const PatchDev*>(B.pd);
+        const SynthParams& sp = *reinterpret_cast<const SynthParams*>(B.spd);
+        // ---- the batch's passes of this part.  Invariant at a pass's
+        // start: if this thread has a candidate in it (c0 + tid < c1),
+        // its record is on the way into slot k (the last commit group).
+        Pass P = first_pass_from(B, 0);
+        if (!fetched) {
+            fetch_first(S.raw[k], B, P, tid);
             cp_async_commit();
+        }
+        fetched = false;
+        bool built = false;     // the next batch
+        {
             while (P.s >= 0) {
                 const int s = P.s;
-                const int t = S.sgb[s];
-                const int b = b_begin + t;
-                const int R = S.mR[t];
-                float2* const ph = S.ph[s & 1];
-                const float bound = 1.001f * (float)(P.c1 - P.c0) * S.mamax[t];   // >= every |S_ij| of the pass
-                const float scale = 1073741824.f / bound;                        // 2^30 / bound
-                const float inv = bound * (1.f / 1073741824.f);                  // 1 / scale
+                const int R = B.sgR[s];
+                // Q16.16 centres of the tile's first texel
+                const int32_t X0 = B.tx0 * kQs + kHalfs, Y0 = B.ty0 * kQs + kHalfs;
+                const float bound = 1.001f * (float)(P.c1 - P.c0) * B.sgA[s];   // >= every |S_ij| of the pass
+                const float scale = 1073741824.f / bound;                      // 2^30 / bound
                 if (tid == 0) atomicAdd(p.stats + 5 + p.nb, (unsigned long long)(P.c1 - P.c0));
-                const Pass Pn = next_pass(S, P, nseg, K, part);
-                const bool pre = Pn.s >= 0 && Pn.c0 + tid < Pn.c1;   // a candidate in the next pass
+                const Pass Pn = next_pass(B, P);
+                // the next pass, or the first of the next batch where that is built
+                fetched = Pn.s < 0 && built;
+                const Batch& Bf = S.bt[fetched ? cur ^ 1 : cur];
+                const Pass Pf = !fetched                ? Pn
+                                : Bf.item < n_items ? first_pass_from(Bf, 0)
+                                                    : Pass{-1, 0, 0};
                 // the (0, 0) corner, shared by every bump whose box starts at
                 // the tile's first texel in both axes: per-thread sums
                 uint32_t z[kPlanes];
 #pragma unroll
                 for (int q = 0; q < kPlanes; ++q) z[q] = 0u;
+                bool hz = false;
                 if (P.c0 + tid >= P.c1) {   // none here: the next pass's first copy
-                    if (pre) fetch_rows(S, p.rec, S.sgrb[Pn.s], S.sgrb[Pn.s + 1] - 1, Pn.c0 + tid, k, tid);
+                    fetch_first(S.raw[k], Bf, Pf, tid);
                     cp_async_commit();
                 }
                 // the row of this thread's next candidate is at or after that of its current one
-                int q = S.sgrb[s];
-                const int qe = S.sgrb[s + 1] - 1;
+                int q = B.sgrb[s];
+                const int qe = B.sgrb[s + 1] - 1;
                 for (int j = P.c0 + tid; j < P.c1; j += kSatThreads) {
                     // the copy of this thread's next candidate starts now
                     if (j + kSatThreads < P.c1)
-                        q = fetch_rows(S, p.rec, q, qe, j + kSatThreads, k ^ 1, tid);
-                    else if (pre)
-                        fetch_rows(S, p.rec, S.sgrb[Pn.s], S.sgrb[Pn.s + 1] - 1, Pn.c0 + tid, k ^ 1, tid);
+                        q = fetch_rows(S.raw[k ^ 1], B, q, qe, j + kSatThreads, tid);
+                    else
+                        fetch_first(S.raw[k ^ 1], Bf, Pf, tid);
                     cp_async_commit();
                     cp_async_wait_prev();   // this candidate's record has landed
                     const BumpRec rc = read_slot(S, k, tid);
@@ -415,6 +493,7 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                         if (a == 0 && c == 0) {
 #pragma unroll
                             for (int q = 0; q < kPlanes; ++q) z[q] += w[q];
+                            hz = true;
                         } else {
                             event9(S, a, c, w, false);
                         }
@@ -424,12 +503,14 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                     }
                 }
                 // (all threads converge here: one reduction per warp and pass)
+                if (__any_sync(0xffffffffu, hz)) {
 #pragma unroll
-                for (int q = 0; q < kPlanes; ++q) z[q] = __reduce_add_sync(0xffffffffu, z[q]);
-                if (lane == 0) {
+                    for (int q = 0; q < kPlanes; ++q) z[q] = __reduce_add_sync(0xffffffffu, z[q]);
+                    if (lane == 0) {
 #pragma unroll
-                    for (int q = 0; q < kPlanes; ++q)
-                        if (z[q]) atomicAdd(&S.E[q][0], z[q]);
+                        for (int q = 0; q < kPlanes; ++q)
+                            if (z[q]) atomicAdd(&S.E[q][0], z[q]);
+                    }
                 }
                 __syncthreads();   // E holds the pass's events
                 if (tid < kScanThreads) {
@@ -458,8 +539,13 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 } else if (tid < kScanThreads + 2 * kT) {
                     // ---- meanwhile spare warps fetch this bucket's texel phases
                     const int h = tid - kScanThreads;
-                    ph[h] = p.phase[(size_t)b * p.phase_len + (h < kT ? ty0 + h : tx0 + (h - kT))];
+                    S.ph[h] = p.phase[(size_t)B.sgb[s] * p.phase_len + (h < kT ? B.ty0 + h : B.tx0 + (h - kT))];
+                } else if (warp >= kBuildWarp0 && !built && (Pn.s < 0 || next_pass(B, Pn).s < 0)) {
+                    // ---- and the builders prepare the next batch, as late as its first
+                    // copies allow (a ticket taken early is work other CTAs cannot take)
+                    build_batch(S, cur ^ 1, !B.last, items, n_items, pdevs, sps, queue, tid - 32 * kBuildWarp0);
                 }
+                built = built || Pn.s < 0 || next_pass(B, Pn).s < 0;
                 __syncthreads();
                 if (tid < kScanThreads) {
                     // ---- prefix along y: one column of one plane per thread.
@@ -490,8 +576,9 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 // zeroed once read (the next pass starts from a cleared array).
                 // Row r > 0 of the segment: the prefix sum of row r - 1 plus
                 // the x prefix of row r (exact modulo 2^32)
-                const float2 ux = ph[kT + cx];   // (cos a_X, sin a_X) of this column
-                const float kh = 0.25f * inv, kd = lamq * inv;
+                const float2 ux = S.ph[kT + cx];   // (cos a_X, sin a_X) of this column
+                const float inv = bound * (1.f / 1073741824.f);                  // 1 / scale
+                const float kh = 0.25f * inv, kd = 0.5f * sp.lam_half * inv;      // (lam / 4)
                 uint32_t sy[kPlanes];
 #pragma unroll
                 for (int r = 0; r < kSegRows; ++r) {
@@ -505,7 +592,7 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                         f[k] = (float)(int32_t)sy[k];
                         S.E[k][o] = 0u;
                     }
-                    const float2 vy = ph[y];   // (cos a_Y, sin a_Y)
+                    const float2 vy = S.ph[y];   // (cos a_Y, sin a_Y)
                     float tt[3], tp[3];
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
@@ -520,27 +607,35 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 P = Pn;
             }
         }
+        if (!built) {   // no pass in this batch
+            __syncthreads();
+            if (warp >= kBuildWarp0)
+                build_batch(S, cur ^ 1, !B.last, items, n_items, pdevs, sps, queue, tid - 32 * kBuildWarp0);
+            __syncthreads();
+        }
 
-        // ---- store: the item's partial plane, or (one plane) the blended maps
-        const int x = tx0 + cx;
-        if (x < sp.W) {
-            const int pitch = G * K > 1 ? partial_pitch(sp.W) : sp.W;
+        // ---- the item done: its partial plane, or (one plane) the blended maps
+        const int x = B.tx0 + cx;
+        if (B.last && x < sp.W) {
+            const bool part_plane = B.planes > 1;
+            const int pitch = part_plane ? partial_pitch(sp.W) : sp.W;
             const size_t plane = (size_t)pitch * sp.H;
-            const int pl = g * K + part;
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
-                float* const dst =
-                    (G * K > 1 ? p.partial + ((size_t)pl * 3 + f) * plane : p.out + (size_t)f * plane) + x;
+                float* const dst = (part_plane ? p.partial + ((size_t)B.plane * 3 + f) * plane : p.out + (size_t)f * plane) + x;
 #pragma unroll
                 for (int r = 0; r < kSegRows; ++r) {
-                    const int y = ty0 + sg * kSegRows + r;
+                    const int y = B.ty0 + sg * kSegRows + r;
                     const float v = f == 0 ? ah[r] : (f == 1 ? adx[r] : ady[r]);
-                    if (y < sp.H) dst[(size_t)y * pitch] = G * K > 1 ? v : blend1(sp, x, y, f, v);
+                    if (y < sp.H) dst[(size_t)y * pitch] = part_plane ? v : blend1(sp, x, y, f, v);
                 }
             }
         }
-        if (tid == 0) S.item = (int)atomicAdd(queue, 1u);
-        __syncthreads();   // the next item's ticket
+        if (B.last) {
+#pragma unroll
+            for (int r = 0; r < kSegRows; ++r) ah[r] = adx[r] = ady[r] = 0.f;
+        }
+        cur ^= 1;
     }
     // the last CTA out resets the queue for the next launch: every CTA takes
     // its last ticket before it counts itself out
