@@ -96,6 +96,7 @@ struct scwp_ctx {
     scwp_spectrum_desc d{};
     std::vector<double> edges;
     cudaStream_t st = nullptr;
+    int device = -1;                  // the device the context was made on
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::string err;
@@ -779,6 +780,10 @@ scwp_status scwp_create(const scwp_spectrum_desc* desc, scwp_ctx** out) {
     if (desc->bucket_edges) ctx->edges.assign(desc->bucket_edges, desc->bucket_edges + desc->n_buckets + 1);
     ctx->d.bucket_edges = nullptr;
     ctx->st = (cudaStream_t)desc->stream;
+    if (cudaGetDevice(&ctx->device) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->device = -1;
+    }
     model_from_desc(ctx->d, ctx->sm);
     auto bail = [&](scwp_status st) {
         scwp_destroy(ctx);
@@ -1607,6 +1612,25 @@ scwp_status scwp_autotune(scwp_ctx* ctx, int32_t reps, int32_t force, scwp_tune_
     return SCWP_OK;
 }
 
+// A map to the caller's device buffer: by a kernel where the buffer lies on
+// this context's device and that device is current, else (another device's
+// memory, managed or mapped memory, anything that is no device allocation) by
+// the copy API, which takes or refuses it.
+static cudaError_t copy_map(scwp_ctx* ctx, float* dst, const float* src, size_t n) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev == ctx->device && ((uintptr_t)dst & 3u) == 0) {
+        bool here = true;
+        for (const float* q : {dst, dst + n - 1}) {
+            cudaPointerAttributes a{};
+            here = here && cudaPointerGetAttributes(&a, q) == cudaSuccess && a.type == cudaMemoryTypeDevice &&
+                   a.device == dev;
+        }
+        if (here) return launch_copy(src, dst, n, ctx->st);
+    }
+    cudaGetLastError();
+    return cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToDevice, ctx->st);
+}
+
 scwp_status scwp_height_map(scwp_ctx* ctx, int32_t patch_id, int32_t field, float* dst, size_t dst_elems,
                             int32_t dst_on_device) {
     scwp_status s = ready(ctx);
@@ -1625,7 +1649,7 @@ scwp_status scwp_height_map(scwp_ctx* ctx, int32_t patch_id, int32_t field, floa
     }
     if (dst_elems < n) return fail(ctx, SCWP_E_INVALID, "dst too small");
     if (dst_on_device) {
-        CU(cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToDevice, ctx->st));
+        CU(copy_map(ctx, dst, src, n));
     } else {
         CU(cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToHost, ctx->st));
         CU(cudaStreamSynchronize(ctx->st));
@@ -1650,7 +1674,7 @@ scwp_status scwp_height_maps(scwp_ctx* ctx, int32_t patch_id, float* dst, size_t
     }
     if (dst_elems < 3 * n) return fail(ctx, SCWP_E_INVALID, "dst too small");
     if (dst_on_device) {
-        CU(cudaMemcpyAsync(dst, src, 3 * n * sizeof(float), cudaMemcpyDeviceToDevice, ctx->st));
+        CU(copy_map(ctx, dst, src, 3 * n));
     } else {
         CU(cudaMemcpyAsync(dst, src, 3 * n * sizeof(float), cudaMemcpyDeviceToHost, ctx->st));
         CU(cudaStreamSynchronize(ctx->st));

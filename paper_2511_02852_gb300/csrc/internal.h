@@ -266,6 +266,9 @@ int synth_tc_ctas_per_sm();
 // unit normals [3][H][W] of the displaced surface of maps [3][H][W] (h, Dx, Dy)
 cudaError_t launch_normals(const float* maps, int W, int H, float cell, float* dst, cudaStream_t st);
 
+// n floats from src to dst, both on the current device
+cudaError_t launch_copy(const float* src, float* dst, size_t n, cudaStream_t st);
+
 // group sums and blend of `n_spans` spans of any patches, one launch
 cudaError_t launch_blend_spans(const BlendSpan* spans, int n_spans, const PatchDev* pdevs, const SynthParams* sps,
                                cudaStream_t st);
