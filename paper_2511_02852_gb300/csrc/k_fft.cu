@@ -11,8 +11,10 @@
 // k_y reads h0 rows k_y and -k_y once each and w(k) (even in k) once, and
 // transforms three rows: H~, D~x, D~y.  The column pass (along y) rebuilds
 // the rows k_y > N/2 by conjugation and packs the real results two to a
-// complex transform: Z = H1 + i Dx1 gives h + i Dx of a column; W = Dy1(x) +
-// i Dy1(x + 1) gives Dy of two columns.  That is 1.5 complex transforms of
+// complex transform: Z = F1(x) + i F1(x + 1), F one of H, Dx, Dy, gives that
+// field of two neighbouring columns, so that a block's columns are neighbours
+// in one plane and every run it reads or writes is a whole number of 32-byte
+// sectors.  That is 1.5 complex transforms of
 // length N per row and per column, and an intermediate of 3 x (N/2 + 1) x N
 // complex values.
 //
@@ -62,7 +64,7 @@ template <int N>
 __host__ __device__ constexpr int threads_per_transform() { return N >= 16 ? N / 16 : 1; }
 template <int N>
 __host__ __device__ constexpr int padded() { return N + N / 16; }
-// columns per column-pass CTA for h + i Dx (twice as many for Dy, in pairs)
+// transforms (column pairs) per column-pass CTA
 template <int N>
 __host__ __device__ constexpr int col_group() { return N >= 2048 ? 4 : N >= 1024 ? 8 : N >= 32 ? 16 : N / 2; }
 // stride of one transform in shared memory: the padded length, rounded to
@@ -341,11 +343,10 @@ __global__ void __launch_bounds__(3 * threads_per_transform<N>(), N >= 4096 ? 1 
     }
 }
 
-// Columns pass.  Blocks 0 .. N/CZ - 1: columns x0 .. x0 + CZ - 1 of h and Dx
-// (one transform Z = H1 + i Dx1 per column); blocks N/CZ .. : columns
-// x0 .. x0 + 2 CZ - 1 of Dy (one transform W = Dy1(x) + i Dy1(x + 1) per
-// column pair).  The rows k_y > N/2 of H1, Dx1 and Dy1 are the conjugates of
-// the rows N - k_y.  out is [3][N][N] (h, Dx, Dy), row-major.
+// Columns pass.  Block: columns x0 .. x0 + 2 CZ - 1 of field blockIdx.x /
+// (N / 2 CZ), one transform Z = F1(x) + i F1(x + 1) per column pair.  The rows
+// k_y > N/2 of F1 are the conjugates of the rows N - k_y.  out is [3][N][N]
+// (h, Dx, Dy), row-major.
 template <int N, int M>
 __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
                                   col_group<N>() * threads_per_transform<N>() <= 512 ? 2 : 1)
@@ -357,10 +358,12 @@ __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
     float2 (*buf)[Np] = reinterpret_cast<float2 (*)[Np]>(smem_cols);   // [CZ][Np]
     pdl_enter();
     const size_t rows = (size_t)(N / 2 + 1) * N;
-    const bool dy = (int)blockIdx.x >= N / CZ;
-    const int x0 = dy ? ((int)blockIdx.x - N / CZ) * 2 * CZ : (int)blockIdx.x * CZ;
-    // load: element (k_y, c) with c fastest (CZ consecutive columns of a
-    // row), every load of the thread issued before the first store
+    constexpr int GF = N / (2 * CZ);   // blocks per field
+    const int field = (int)blockIdx.x / GF;
+    const int x0 = ((int)blockIdx.x - field * GF) * 2 * CZ;
+    const float2* const src = bg.I + field * rows + x0;
+    // load: element (k_y, c) with c fastest (CZ consecutive column pairs of
+    // a row), every load of the thread issued before the first store
     constexpr int E = ((N / 2 + 1) * CZ + NT - 1) / NT;
     float4 ld[E];
 #pragma unroll
@@ -368,12 +371,7 @@ __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
         const int w = threadIdx.x + i * NT;
         if (w < (N / 2 + 1) * CZ) {
             const int m = w / CZ, c = w - m * CZ;
-            if (!dy) {
-                const float2 h = bg.I[(size_t)m * N + x0 + c], d = bg.I[rows + (size_t)m * N + x0 + c];
-                ld[i] = make_float4(h.x, h.y, d.x, d.y);
-            } else {
-                ld[i] = *reinterpret_cast<const float4*>(&bg.I[2 * rows + (size_t)m * N + x0 + 2 * c]);
-            }
+            ld[i] = *reinterpret_cast<const float4*>(&src[(size_t)m * N + 2 * c]);
         }
     }
 #pragma unroll
@@ -381,8 +379,8 @@ __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
         const int w = threadIdx.x + i * NT;
         if (w >= (N / 2 + 1) * CZ) continue;
         const int m = w / CZ, c = w - m * CZ;
-        // (p, q) = (H1, Dx1) or (Dy1(x), Dy1(x + 1)): the transform's rows m
-        // and N - m are p + i q and conj(p) + i conj(q)
+        // (p, q) = (F1(x), F1(x + 1)): the transform's rows m and N - m
+        // are p + i q and conj(p) + i conj(q)
         const float4 pq = ld[i];
         buf[c][pad(m)] = make_float2(pq.x - pq.w, pq.y + pq.z);
         if (m > 0 && m < N / 2) buf[c][pad(N - m)] = make_float2(pq.x + pq.w, pq.z - pq.y);
@@ -390,19 +388,17 @@ __global__ void __launch_bounds__(col_group<N>() * threads_per_transform<N>(),
     __syncthreads();
     const int t = threadIdx.x / P, jt = threadIdx.x % P;
     fft_inv<N>(buf[t], jt, bg.tw);
-    const size_t plane = (size_t)N * N;
-    if (!dy) {
-        for (int w = threadIdx.x; w < N * CZ; w += NT) {
-            const int y = w / CZ, c = w - y * CZ;
-            const float2 v = buf[c][pad(y)];
-            bg.out[(size_t)y * N + x0 + c] = v.x;
-            bg.out[plane + (size_t)y * N + x0 + c] = v.y;
-        }
-    } else {
-        for (int w = threadIdx.x; w < N * CZ; w += NT) {
-            const int y = w / CZ, c = w - y * CZ;
-            const float2 v = buf[c][pad(y)];
-            *reinterpret_cast<float2*>(&bg.out[2 * plane + (size_t)y * N + x0 + 2 * c]) = v;
+    float* const dst = bg.out + (size_t)field * N * N + x0;
+    const bool whole = ((uintptr_t)bg.out & 7u) == 0;   // a caller's own output may start on any float
+    for (int w = threadIdx.x; w < N * CZ; w += NT) {
+        const int y = w / CZ, c = w - y * CZ;
+        const float2 v = buf[c][pad(y)];
+        float* const o = dst + (size_t)y * N + 2 * c;
+        if (whole) {
+            *reinterpret_cast<float2*>(o) = v;
+        } else {
+            o[0] = v.x;
+            o[1] = v.y;
         }
     }
 }
@@ -429,7 +425,7 @@ cudaError_t launch_n(const BgPack<M>& pk, int m, cudaStream_t st, const float2* 
     cudaError_t e;
     e = launch_pdl(k_spectrum_rows<N, M>, dim3(N / 2 + 1, m), 3 * P, smr, st, pk, t_dev);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_fft_cols<N, M>, dim3(N / CZ + N / (2 * CZ), m), CZ * P, smc, st, pk);
+    e = launch_pdl(k_fft_cols<N, M>, dim3(3 * (N / (2 * CZ)), m), CZ * P, smc, st, pk);
     count_launches(2);
     return e;
 }
