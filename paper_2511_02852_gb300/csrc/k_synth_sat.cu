@@ -89,7 +89,7 @@ static_assert(kScanThreads % 32 == 0, "whole scan warps");
 
 constexpr int kBuildWarp0 = 24;              // warps 24 .. 31 build the next batch
 constexpr int kBuildThreads = kSatThreads - 32 * kBuildWarp0;
-static_assert(kScanThreads + 2 * kT <= 32 * kBuildWarp0, "phase threads and builders apart");
+static_assert(kScanThreads + 2 * kT + 32 <= 32 * kBuildWarp0, "phase threads and builders apart");
 
 // A batch of one item: segments (bucket, row range) whose bin rows fit the row table.
 struct Batch {
@@ -106,10 +106,29 @@ struct Batch {
     alignas(16) unsigned char spd[sizeof(SynthParams)];
 };
 
+// A pass as its threads read it: written once, by one thread, in the y-prefix
+// phase of the pass before (worked out by every warp for itself, it took
+// about 1,000 of a pass's 16,000 cycles).
+struct alignas(16) PassDesc {
+    int32_t s, c0, c1, rb, re;            // segment (kEmpty, kDone: none), candidates, row table rows
+    int32_t R, bucket, batch;
+    int32_t X0, Y0;                       // Q16.16 centre of the tile's first texel
+    float scale, inv;
+    int32_t fetched;                      // its first copies are on their way already
+    int32_t build;                        // its x-prefix phase builds the next batch
+    int32_t built;                        // ... is there after that phase
+    int32_t last;                         // the batch's last pass
+    int32_t f_batch, f_c0, f_c1, f_rb, f_re;   // the pass whose first copies this one starts (f_c0 == f_c1: none)
+};
+constexpr int kEmpty = -1, kDone = -2;    // a batch without a pass; no more items
+constexpr int kDescThread = 32 * kBuildWarp0 - 32;   // a thread of a warp that neither scans nor builds
+
 struct SatSmem {
     uint32_t E[kPlanes][kT * kT];         // difference arrays, then prefix sums; zero between passes
     alignas(128) BumpRec raw[2][kSatThreads];   // two record slots per thread
     alignas(16) float2 ph[2 * kT];        // texel phases (cos, sin) a of the pass's bucket: rows, then columns
+    alignas(16) uint32_t Z[kPlanes][32];  // the (0, 0) corner of the pass, per lane; zero between passes
+    PassDesc pass[2];
     Batch bt[2];
     // the builders' table of the item's buckets, and the segments' first rows
     int32_t mR[kMaxBuckets], mnbx[kMaxBuckets], mbase[kMaxBuckets];
@@ -128,10 +147,10 @@ __device__ __forceinline__ int sw(int y, int x) { return y * kT + (x ^ (y & 31))
 __device__ __forceinline__ int clamp_t(int t) { return min(max(t, 0), kT); }
 
 // the nine components of one corner event
-__device__ __forceinline__ void event9(SatSmem& S, int x, int y, const uint32_t (&w)[kPlanes], bool neg) {
+__device__ __forceinline__ void event9(SatSmem& S, int x, int y, const uint32_t (&w)[kPlanes]) {
     const int o = sw(y, x);
 #pragma unroll
-    for (int k = 0; k < kPlanes; ++k) atomicAdd(&S.E[k][o], neg ? 0u - w[k] : w[k]);
+    for (int k = 0; k < kPlanes; ++k) atomicAdd(&S.E[k][o], w[k]);
 }
 
 // inclusive warp scan of v
@@ -195,31 +214,84 @@ __device__ __forceinline__ Pass next_pass(const Batch& B, Pass P) {
     return first_pass_from(B, P.s + 1);
 }
 
-// This thread's copy of candidate j (of the segment whose table rows are
-// [lo, hi]) into its slot; returns the candidate's row.  The row is the last
-// one that starts at or before j (empty rows start where the next one does).
-__device__ __forceinline__ int fetch_rows(BumpRec* slot, const Batch& B, int lo, int hi, int j, int tid) {
-    if (lo < hi && B.cum[lo + 1] > j) hi = lo;   // still the row of the hint
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (B.cum[mid] <= j)
-            lo = mid;
-        else
-            hi = mid - 1;
+// This thread's copy of candidate j0 + lane (if below c1) of the segment whose
+// table rows are [qb, re) into its slot; qb moves on to the row of j0.  A
+// candidate's row is the last one that starts at or before it (empty rows
+// start where the next one does): the warp finds that of its first candidate
+// with one load and a ballot per 32 rows, each lane steps on from there (a
+// bisection per lane took twice the instructions).
+__device__ __forceinline__ void fetch(BumpRec* slot, const Batch& B, int& qb, int re, int j0, int c1, int tid) {
+    const int lane = tid & 31;
+    for (;;) {
+        const unsigned m = __ballot_sync(0xffffffffu, qb + lane < re && B.cum[qb + lane] <= j0);
+        if (m != 0xffffffffu) {   // (the rows that start at or before j0 come first)
+            qb += __popc(m) - 1;
+            break;
+        }
+        qb += 32;
     }
-    const BumpRec* const rec = reinterpret_cast<const PatchDev*>(B.pd)->rec;
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(rec + B.rs[lo] + (j - B.cum[lo]));
-    unsigned char* dst = reinterpret_cast<unsigned char*>(slot + tid);
-    const int hs = half_swap(tid);
-    cp_async16(dst + 16 * hs, src);
-    cp_async16(dst + 16 * (hs ^ 1), src + 16);
-    return lo;
+    const int j = j0 + lane;
+    if (j < c1) {
+        int r = qb;
+        while (r + 1 < re && B.cum[r + 1] <= j) ++r;
+        const BumpRec* const rec = reinterpret_cast<const PatchDev*>(B.pd)->rec;
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(rec + B.rs[r] + (j - B.cum[r]));
+        unsigned char* dst = reinterpret_cast<unsigned char*>(slot + tid);
+        const int hs = half_swap(tid);
+        cp_async16(dst + 16 * hs, src);
+        cp_async16(dst + 16 * (hs ^ 1), src + 16);
+    }
 }
 
-// ... of this thread's first candidate of pass P, if it has one
-__device__ __forceinline__ void fetch_first(BumpRec* slot, const Batch& B, Pass P, int tid) {
-    if (P.s >= 0 && P.c0 + tid < P.c1)
-        fetch_rows(slot, B, B.sgrb[P.s], B.sgrb[P.s + 1] - 1, P.c0 + tid, tid);
+// Pass P of batch b into D.  built: the batch after it is built (so that P can
+// start the copies of that one's first pass).  One thread.
+__device__ void describe(SatSmem& S, PassDesc& D, int b, Pass P, bool fetched, bool built, int n_items) {
+    const Batch& B = S.bt[b];
+    D.batch = b;
+    D.s = P.s;
+    D.last = 1;
+    if (P.s < 0) {
+        D.s = kEmpty;
+        return;
+    }
+    const float bound = 1.001f * (float)(P.c1 - P.c0) * B.sgA[P.s];   // >= every |S_ij| of the pass
+    D.scale = 1073741824.f / bound;                                  // 2^30 / bound
+    D.inv = bound * (1.f / 1073741824.f);                            // 1 / scale
+    D.c0 = P.c0;
+    D.c1 = P.c1;
+    D.rb = B.sgrb[P.s];
+    D.re = B.sgrb[P.s + 1];
+    D.R = B.sgR[P.s];
+    D.bucket = B.sgb[P.s];
+    D.X0 = B.tx0 * kQs + kHalfs;
+    D.Y0 = B.ty0 * kQs + kHalfs;
+    D.fetched = fetched;
+    const Pass Pn = next_pass(B, P);
+    D.last = Pn.s < 0;
+    // the next batch, as late as its first copies allow (a ticket taken early
+    // is work other CTAs cannot take)
+    D.build = !built && (Pn.s < 0 || next_pass(B, Pn).s < 0);
+    D.built = built || D.build;
+    Pass Pf = Pn;
+    D.f_batch = b;
+    if (Pn.s < 0 && built) {
+        D.f_batch = b ^ 1;
+        if (S.bt[b ^ 1].item < n_items) Pf = first_pass_from(S.bt[b ^ 1], 0);
+    }
+    const Batch& Bf = S.bt[D.f_batch];
+    D.f_c0 = Pf.s < 0 ? 0 : Pf.c0;
+    D.f_c1 = Pf.s < 0 ? 0 : Pf.c1;
+    D.f_rb = Pf.s < 0 ? 0 : Bf.sgrb[Pf.s];
+    D.f_re = Pf.s < 0 ? 0 : Bf.sgrb[Pf.s + 1];
+}
+
+// The first pass of batch b into D.
+__device__ void describe_first(SatSmem& S, PassDesc& D, int b, bool fetched, int n_items) {
+    if (S.bt[b].item >= n_items) {
+        D.s = kDone;
+        return;
+    }
+    describe(S, D, b, first_pass_from(S.bt[b], 0), fetched, false, n_items);
 }
 
 __device__ __forceinline__ void builders_sync() {
@@ -409,69 +481,71 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
         const int bt = tid - 32 * kBuildWarp0;
         if (bt < 2) S.bt[bt].patch = -1;
         build_batch(S, 0, false, items, n_items, pdevs, sps, queue, bt);
-    } else {   // E starts zeroed, and every pass leaves it zeroed again
+    } else {   // E and Z start zeroed, and every pass leaves them zeroed again
         uint4* e4 = reinterpret_cast<uint4*>(&S.E[0][0]);
         for (int k = tid; k < kPlanes * kT * kT / 4; k += 32 * kBuildWarp0) e4[k] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid < kPlanes * 32) (&S.Z[0][0])[tid] = 0u;
     }
+    __syncthreads();
+    if (tid == kDescThread) describe_first(S, S.pass[0], 0, false, n_items);
     __syncthreads();
     float ah[kSegRows], adx[kSegRows], ady[kSegRows];
 #pragma unroll
     for (int r = 0; r < kSegRows; ++r) ah[r] = adx[r] = ady[r] = 0.f;
-    int cur = 0, k = 0;         // the batch; the record slot of the next candidate
-    bool fetched = false;       // the batch's first copies are on their way
-    while (S.bt[cur].item < n_items) {
-        const Batch& B = S.bt[cur];
+    int dp = 0, k = 0;          // the pass's description; the record slot of the next candidate
+    for (;;) {
+        const PassDesc& D = S.pass[dp];
+        if (D.s == kDone) break;
+        const Batch& B = S.bt[D.batch];
         const PatchDev& p = *reinterpret_cast<const PatchDev*>(B.pd);
         const SynthParams& sp = *reinterpret_cast<const SynthParams*>(B.spd);
-        // ---- the batch's passes of this part.  Invariant at a pass's
-        // start: if this thread has a candidate in it (c0 + tid < c1),
-        // its record is on the way into slot k (the last commit group).
-        Pass P = first_pass_from(B, 0);
-        if (!fetched) {
-            fetch_first(S.raw[k], B, P, tid);
-            cp_async_commit();
-        }
-        fetched = false;
-        bool built = false;     // the next batch
-        {
-            while (P.s >= 0) {
-                const int s = P.s;
-                const int R = B.sgR[s];
-                // Q16.16 centres of the tile's first texel
-                const int32_t X0 = B.tx0 * kQs + kHalfs, Y0 = B.ty0 * kQs + kHalfs;
-                const float bound = 1.001f * (float)(P.c1 - P.c0) * B.sgA[s];   // >= every |S_ij| of the pass
-                const float scale = 1073741824.f / bound;                      // 2^30 / bound
-                if (tid == 0) atomicAdd(p.stats + 5 + p.nb, (unsigned long long)(P.c1 - P.c0));
-                const Pass Pn = next_pass(B, P);
-                // the next pass, or the first of the next batch where that is built
-                fetched = Pn.s < 0 && built;
-                const Batch& Bf = S.bt[fetched ? cur ^ 1 : cur];
-                const Pass Pf = !fetched                ? Pn
-                                : Bf.item < n_items ? first_pass_from(Bf, 0)
-                                                    : Pass{-1, 0, 0};
+        if (D.s == kEmpty) {
+            __syncthreads();
+            if (warp >= kBuildWarp0)
+                build_batch(S, D.batch ^ 1, !B.last, items, n_items, pdevs, sps, queue, tid - 32 * kBuildWarp0);
+            __syncthreads();
+            if (tid == kDescThread) describe_first(S, S.pass[dp ^ 1], D.batch ^ 1, false, n_items);
+            __syncthreads();
+        } else {
+            {
+                // ---- the pass's events.  Invariant from here on: if this
+                // thread has a candidate (c0 + tid < c1), its record is on
+                // the way into slot k (the last commit group).
+                const int c1 = D.c1, R = D.R;
+                const int32_t X0 = D.X0, Y0 = D.Y0;
+                const float scale = D.scale;
+                int j0 = D.c0 + 32 * warp, q = D.rb;   // the warp's next candidates and a row at or before theirs
+                if (!D.fetched) {
+                    if (j0 < c1) fetch(S.raw[k], B, q, D.re, j0, c1, tid);
+                    cp_async_commit();
+                }
+                // the copies of the next pass's first candidates, once this warp has no more of its own
+                auto fetch_next = [&](int slot) {
+                    const int jf = D.f_c0 + 32 * warp;
+                    int qf = D.f_rb;
+                    if (jf < D.f_c1) fetch(S.raw[slot], S.bt[D.f_batch], qf, D.f_re, jf, D.f_c1, tid);
+                };
                 // the (0, 0) corner, shared by every bump whose box starts at
                 // the tile's first texel in both axes: per-thread sums
                 uint32_t z[kPlanes];
 #pragma unroll
                 for (int q = 0; q < kPlanes; ++q) z[q] = 0u;
                 bool hz = false;
-                if (P.c0 + tid >= P.c1) {   // none here: the next pass's first copy
-                    fetch_first(S.raw[k], Bf, Pf, tid);
+                if (j0 >= c1) {
+                    fetch_next(k);
                     cp_async_commit();
                 }
-                // the row of this thread's next candidate is at or after that of its current one
-                int q = B.sgrb[s];
-                const int qe = B.sgrb[s + 1] - 1;
-                for (int j = P.c0 + tid; j < P.c1; j += kSatThreads) {
+                for (; j0 < c1; j0 += kSatThreads) {   // (uniform over the warp)
                     // the copy of this thread's next candidate starts now
-                    if (j + kSatThreads < P.c1)
-                        q = fetch_rows(S.raw[k ^ 1], B, q, qe, j + kSatThreads, tid);
+                    if (j0 + kSatThreads < c1)
+                        fetch(S.raw[k ^ 1], B, q, D.re, j0 + kSatThreads, c1, tid);
                     else
-                        fetch_first(S.raw[k ^ 1], Bf, Pf, tid);
+                        fetch_next(k ^ 1);
                     cp_async_commit();
                     cp_async_wait_prev();   // this candidate's record has landed
                     const BumpRec rc = read_slot(S, k, tid);
                     k ^= 1;
+                    if (j0 + lane >= c1) continue;
                     // texel t of the tile is inside iff x_b - R < X0 + t Q < x_b + R
                     const int a = clamp_t(((rc.x - R - X0) >> 16) + 1);
                     const int bb = clamp_t(-((X0 - rc.x - R) >> 16));
@@ -495,22 +569,22 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                             for (int q = 0; q < kPlanes; ++q) z[q] += w[q];
                             hz = true;
                         } else {
-                            event9(S, a, c, w, false);
+                            event9(S, a, c, w);
                         }
-                        if (bb < kT) event9(S, bb, c, w, true);
-                        if (d < kT) event9(S, a, d, w, true);
-                        if (bb < kT && d < kT) event9(S, bb, d, w, false);
+                        if (bb < kT && d < kT) event9(S, bb, d, w);
+#pragma unroll
+                        for (int q = 0; q < kPlanes; ++q) w[q] = 0u - w[q];
+                        if (bb < kT) event9(S, bb, c, w);
+                        if (d < kT) event9(S, a, d, w);
                     }
                 }
-                // (all threads converge here: one reduction per warp and pass)
+                // the (0, 0) corner by lane: 32 different banks, where one
+                // reduction per warp and plane and an add to nine shared words
+                // took 1,100 cycles a pass
+                __syncwarp();
                 if (__any_sync(0xffffffffu, hz)) {
 #pragma unroll
-                    for (int q = 0; q < kPlanes; ++q) z[q] = __reduce_add_sync(0xffffffffu, z[q]);
-                    if (lane == 0) {
-#pragma unroll
-                        for (int q = 0; q < kPlanes; ++q)
-                            if (z[q]) atomicAdd(&S.E[q][0], z[q]);
-                    }
+                    for (int q = 0; q < kPlanes; ++q) atomicAdd(&S.Z[q][lane], z[q]);
                 }
                 __syncthreads();   // E holds the pass's events
                 if (tid < kScanThreads) {
@@ -522,6 +596,15 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                     uint32_t cr[4], nx[4], run = 0u;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) cr[k] = E[sw(y, k)];
+                    if (y == 0) {   // the (0, 0) corner's sum
+                        uint4* const Z4 = reinterpret_cast<uint4*>(S.Z[tid / kT]);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const uint4 v = Z4[k];
+                            run += (v.x + v.y) + (v.z + v.w);
+                            Z4[k] = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
 #pragma unroll
                     for (int x0 = 0; x0 < kT; x0 += 4) {
                         if (x0 + 4 < kT) {
@@ -539,13 +622,10 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 } else if (tid < kScanThreads + 2 * kT) {
                     // ---- meanwhile spare warps fetch this bucket's texel phases
                     const int h = tid - kScanThreads;
-                    S.ph[h] = p.phase[(size_t)B.sgb[s] * p.phase_len + (h < kT ? B.ty0 + h : B.tx0 + (h - kT))];
-                } else if (warp >= kBuildWarp0 && !built && (Pn.s < 0 || next_pass(B, Pn).s < 0)) {
-                    // ---- and the builders prepare the next batch, as late as its first
-                    // copies allow (a ticket taken early is work other CTAs cannot take)
-                    build_batch(S, cur ^ 1, !B.last, items, n_items, pdevs, sps, queue, tid - 32 * kBuildWarp0);
+                    S.ph[h] = p.phase[(size_t)D.bucket * p.phase_len + (h < kT ? B.ty0 + h : B.tx0 + (h - kT))];
+                } else if (warp >= kBuildWarp0 && D.build) {   // ---- and the builders prepare the next batch
+                    build_batch(S, D.batch ^ 1, !B.last, items, n_items, pdevs, sps, queue, tid - 32 * kBuildWarp0);
                 }
-                built = built || Pn.s < 0 || next_pass(B, Pn).s < 0;
                 __syncthreads();
                 if (tid < kScanThreads) {
                     // ---- prefix along y: one column of one plane per thread.
@@ -570,6 +650,12 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
 #pragma unroll
                         for (int k = 0; k < 4; ++k) cr[k] = nx[k];
                     }
+                } else if (tid == kDescThread) {   // ---- meanwhile one thread describes the next pass
+                    atomicAdd(p.stats + 5 + p.nb, (unsigned long long)(D.c1 - D.c0));
+                    if (D.last)
+                        describe_first(S, S.pass[dp ^ 1], D.batch ^ 1, D.f_batch != D.batch, n_items);
+                    else
+                        describe(S, S.pass[dp ^ 1], D.batch, next_pass(B, Pass{D.s, D.c0, D.c1}), true, D.built, n_items);
                 }
                 __syncthreads();
                 // ---- this thread's texels contracted; each element of E is
@@ -577,7 +663,7 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 // Row r > 0 of the segment: the prefix sum of row r - 1 plus
                 // the x prefix of row r (exact modulo 2^32)
                 const float2 ux = S.ph[kT + cx];   // (cos a_X, sin a_X) of this column
-                const float inv = bound * (1.f / 1073741824.f);                  // 1 / scale
+                const float inv = D.inv;
                 const float kh = 0.25f * inv, kd = 0.5f * sp.lam_half * inv;      // (lam / 4)
                 uint32_t sy[kPlanes];
 #pragma unroll
@@ -604,19 +690,13 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                     ady[r] = fmaf(kd, fmaf(-ux.y, tp[2], fmaf(ux.x, tp[1], tp[0])), ady[r]);
                 }
                 __syncthreads();   // E cleared; the phases may be rewritten
-                P = Pn;
             }
-        }
-        if (!built) {   // no pass in this batch
-            __syncthreads();
-            if (warp >= kBuildWarp0)
-                build_batch(S, cur ^ 1, !B.last, items, n_items, pdevs, sps, queue, tid - 32 * kBuildWarp0);
-            __syncthreads();
         }
 
         // ---- the item done: its partial plane, or (one plane) the blended maps
         const int x = B.tx0 + cx;
-        if (B.last && x < sp.W) {
+        const bool done = D.last && B.last;
+        if (done && x < sp.W) {
             const bool part_plane = B.planes > 1;
             const int pitch = part_plane ? partial_pitch(sp.W) : sp.W;
             const size_t plane = (size_t)pitch * sp.H;
@@ -631,11 +711,11 @@ __global__ void __launch_bounds__(kSatThreads, 1) k_synth_sat(const TcItem* item
                 }
             }
         }
-        if (B.last) {
+        if (done) {
 #pragma unroll
             for (int r = 0; r < kSegRows; ++r) ah[r] = adx[r] = ady[r] = 0.f;
         }
-        cur ^= 1;
+        dp ^= 1;
     }
     // the last CTA out resets the queue for the next launch: every CTA takes
     // its last ticket before it counts itself out
