@@ -13,8 +13,8 @@ workload is the largest single-GPU scene, mixed_large (2048^2 FFT over 4 km,
 batched mode (one synthesis launch over all patches, frames replayed as
 captured CUDA graphs; a one-patch scene launches eagerly, chained by
 programmatic dependent launch) with the summed-area synthesis.  Beside it on
-the same line: the same scene in plain mode (one synthesis launch per
-patch, eager launches), the tensor-core gather, and the metric's "batched vs
+the same line: the same scene in plain mode (eager launches), the
+tensor-core gather, and the metric's "batched vs
 plain" on the 32-patch batched workload (--compare-frames frames in each
 mode).  The metric is particle-pixel (bump-texel) evaluations per second,
 the eval count being the exact integer count of (bump, texel-centre) pairs
@@ -578,8 +578,8 @@ def frame_summary(ms, ev, mode):
 def batched_vs_plain(args, flush, stream, frames):
     """The metric's "batched vs plain" on the 32-patch batched workload: the
     same scene stepped in batched mode (one synthesis launch over every
-    patch, frames replayed as captured CUDA graphs) and in plain mode (one
-    synthesis launch per patch, eager launches), `frames` timed frames each."""
+    patch, frames replayed as captured CUDA graphs) and in plain mode (the same
+    launches, eagerly), `frames` timed frames each."""
     import torch
     from paper_2511_02852_gb300 import scwp
     cfg = workload_config("batched")
@@ -595,7 +595,7 @@ def batched_vs_plain(args, flush, stream, frames):
         torch.cuda.synchronize()
         ms, ev = timed_frames(sc, cfg, frames, flush, stream)
         out[mode] = frame_summary(ms, ev, "one synthesis launch over all 32 patches, captured frame graph"
-                                  if on else "one synthesis launch per patch, eager launches")
+                                  if on else "one synthesis launch over all 32 patches, eager launches")
         out[mode]["autotune"] = tuned
     out["speedup_frames_per_s"] = out["batched"]["frames_per_s"] / out["plain"]["frames_per_s"]
     sc.close()
@@ -679,7 +679,7 @@ def run_ours(args):
         roofline = tc_roofline(sc, cfg, synth_ms, stage_info, args.synth == "fp16")
     roof_fft = fft_roofline(cfg, fft_ms)
 
-    # the same scene in plain mode (one patch per launch, eager launches)
+    # the same scene in plain mode (eager launches)
     plain = None
     if args.batched and not args.no_compare:
         sc.set_batched(False)
@@ -689,7 +689,7 @@ def run_ours(args):
         plain_tune = tune(sc, args, flush, dt)
         ms, ev = timed_frames(sc, cfg, max(10, min(args.steps, 50)), flush, stream)
         sc.set_batched(True)
-        plain = frame_summary(ms, ev, "plain: one synthesis launch per patch, eager launches")
+        plain = frame_summary(ms, ev, "plain: eager launches")
         plain["autotune"] = plain_tune
 
     # the other synthesis on the same scene: the tensor-core gather beside the
@@ -818,7 +818,7 @@ def main():
                     help="one synthesis launch over all patches of the frame, frames replayed as CUDA "
                          "graphs (scwp_set_batched; the default)")
     ap.add_argument("--plain", action="store_true",
-                    help="one synthesis launch per patch, frames launched eagerly")
+                    help="frames launched eagerly, not replayed from a graph")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-tune", action="store_true",
                     help="skip the summed-area autotuner (scwp_autotune) before the timed frames")

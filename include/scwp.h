@@ -323,7 +323,9 @@ scwp_status scwp_set_bucket_range(scwp_ctx* ctx, int32_t b_lo, int32_t b_hi);
  * group-sum blend launch; per-patch bucket-group counts are planned for the
  * whole frame instead of for each patch alone.  The results are the same
  * sums as the one-patch-per-launch path (with another grouping, the same
- * values up to FP32 rounding order).  Applies to SCWP_SYNTH_SAT,
+ * values up to FP32 rounding order).  (SCWP_SYNTH_SAT runs several patches
+ * as one launch in either mode; batched frames of several patches replay a
+ * captured graph.)  Applies to SCWP_SYNTH_SAT,
  * SCWP_SYNTH_GATHER and SCWP_SYNTH_GATHER_FP16; the
  * paper has no counterpart (its frame is one scene on one GPU).  Returns
  * SCWP_E_INVALID for a null context; takes effect at the next synthesis. */
@@ -430,8 +432,8 @@ void scwp_destroy(scwp_ctx* ctx);
  * Each scene is a context of its own (its spectrum, background and patches)
  * created by the server on the server's stream and allocator, in batched
  * mode.  scwp_server_tick takes every scene that has a pending request and
- * no frame in flight, enqueues each one's background and particle stages
- * (on eight internal streams) and runs the synthesis of all of them as ONE
+ * no frame in flight, enqueues the background and particle stages of all of
+ * them (on two internal streams) and runs the synthesis of all of them as ONE
  * launch over the union of their planned (patch, tile, bucket group) items,
  * heaviest first, followed by one group-sum blend launch (one such pair per
  * synthesis mode in use: a scene keeps its context's mode, by default

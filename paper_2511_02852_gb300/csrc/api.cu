@@ -371,11 +371,16 @@ std::vector<double> tile_bucket_stages(const PatchHost& P, int& tiles) {
 }
 
 // Work of the summed-area synthesis per (tile, bucket), in the same stage
-// units: a fixed part (three rounds of clearing, two prefix passes and the
-// 3 x 3 contraction over the tile's texels) plus one part per candidate bump
-// of the bins that reach the tile (its corner events).
-constexpr double kSatBucketUs = 2.0;
-constexpr double kSatBumpUs = 0.0008;
+// units: a fixed part per pass (the prefixes, the contraction and the latency
+// of its events: 11,000 cycles by the kernel's clocks) plus one part per
+// candidate bump of the bins that reach the tile (75 cycles a warp's 32), and
+// per item its start and its store (5,000 cycles).
+constexpr double kSatBucketUs = 5.7;
+constexpr double kSatBumpUs = 0.0012;
+constexpr double kSatItemStages = 2.0;
+// The group-sum blend: its launch, and its planes at the rate it reads them
+constexpr double kBlendUs = 3.0;
+constexpr double kBlendBytesPerUs = 6.0e6;
 
 std::vector<double> tile_bucket_sat(const PatchHost& P, int& tiles, double* max_passes = nullptr) {
     const PatchTablesHost& T = P.T;
@@ -408,8 +413,8 @@ std::vector<double> tile_bucket_sat(const PatchHost& P, int& tiles, double* max_
     return est;
 }
 
-double item_work(const std::vector<double>& est, int nb, int t, int g, int G) {
-    double s = kItemStages;
+double item_work(const std::vector<double>& est, int nb, int t, int g, int G, bool sat = false) {
+    double s = sat ? kSatItemStages : kItemStages;
     for (int i = (g * nb) / G; i < ((g + 1) * nb) / G; ++i) s += est[(size_t)t * nb + i];
     return s;
 }
@@ -442,10 +447,10 @@ std::vector<BlendSpan> blend_spans(const PatchHost& P, int G) {
 // to at most `cap` stages; a part item costs its set-up plus 1/K of the rest.
 int sat_parts_for(double wmax, double cap, int kmax) {
     int K = 1;
-    while (K < kmax && kItemStages + (wmax - kItemStages) / K > cap) ++K;
+    while (K < kmax && kSatItemStages + (wmax - kSatItemStages) / K > cap) ++K;
     return K;
 }
-double part_work(double w, int K) { return kItemStages + (w - kItemStages) / K; }
+double part_work(double w, int K) { return K > 1 ? kSatItemStages + (w - kSatItemStages) / K : w; }
 
 // Plan of one patch launched alone: G minimises the simulated makespan over
 // the device's resident CTA slots plus the traffic of the group-sum blend.
@@ -461,24 +466,21 @@ void plan_patch(PatchHost& P, int slots, bool sat = false, double gmul = 1.0, in
     auto build = [&](int G) {   // the heaviest-first plan with G groups, and its modelled cost
         std::vector<double> work((size_t)tiles * G);
         for (int t = 0; t < tiles; ++t)
-            for (int g = 0; g < G; ++g) work[(size_t)t * G + g] = item_work(est, nb, t, g, G);
+            for (int g = 0; g < G; ++g) work[(size_t)t * G + g] = item_work(est, nb, t, g, G, sat);
         std::vector<int> order(work.size());
         for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
-        const double blend = G > 1 ? (G + 1) * 12.0 * P.T.W * P.T.H / kHbmBytesPerUs : 0.0;
+        const double blend = G <= 1 ? 0.0
+                             : sat  ? kBlendUs + (G + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs
+                                    : (G + 1) * 12.0 * P.T.W * P.T.H / kHbmBytesPerUs;
         std::vector<TcItem> items;
         for (int k : order) items.push_back(TcItem{P.index, k / G, k % G, G});
         return std::make_pair(makespan(work, order, slots) * kStageUs + blend, items);
     };
-    // the summed-area items cost about the same per bucket; the smallest G
-    // that gives three waves over the slots, as far as the buckets allow
     const int gmax = std::max(1, std::min(std::min(nb, 16), gcap));
-    int g_lo = 1;
-    if (sat)
-        while (g_lo < gmax && (double)tiles * g_lo < 3.0 * slots) ++g_lo;
-    for (int G = g_lo; G <= gmax; ++G) {
+    for (int G = 1; G <= gmax; ++G) {
         auto r = build(G);
-        if (G == g_lo || r.first < best_cost) {
+        if (G == 1 || r.first < best_cost) {
             best_cost = r.first;
             groups = G;
             plan.swap(r.second);
@@ -498,7 +500,7 @@ void plan_patch(PatchHost& P, int slots, bool sat = false, double gmul = 1.0, in
         // (the makespan's lower bound), with at most one wave of items
         double total = 0.0, wmax = 0.0;
         for (const TcItem& it : plan) {
-            const double w = item_work(est, nb, it.tile, it.group, groups);
+            const double w = item_work(est, nb, it.tile, it.group, groups, true);
             total += w;
             wmax = std::max(wmax, w);
         }
@@ -508,7 +510,7 @@ void plan_patch(PatchHost& P, int slots, bool sat = false, double gmul = 1.0, in
             std::vector<std::pair<double, TcItem>> parts;
             for (const TcItem& it : plan)
                 for (int q = 0; q < K; ++q)
-                    parts.push_back({part_work(item_work(est, nb, it.tile, it.group, groups), K),
+                    parts.push_back({part_work(item_work(est, nb, it.tile, it.group, groups, true), K),
                                      TcItem{it.patch, it.tile, it.group | (q << 16), groups | (K << 16)}});
             std::stable_sort(parts.begin(), parts.end(),
                              [](const std::pair<double, TcItem>& a, const std::pair<double, TcItem>& b) {
@@ -543,65 +545,91 @@ bool sat3_fits(const PatchHost& P) {
 }
 
 // Plan of all patches in one launch: each patch's G is the smallest that
-// keeps its largest item under a quarter of the average per-slot load, and
-// all items of all patches run heaviest first.
+// keeps its largest item under `share` of the average per-slot load (a
+// quarter for the tensor-core gather), and all items of all patches run
+// heaviest first.  For the summed-area synthesis the share is the one, of a
+// few, with the smallest modelled makespan and blend: an item's start and
+// store cost more than half a pass, so a scene that fits one wave of longer
+// items runs them rather than three of single buckets (a quarter for every
+// scene: a server round of 12 scenes 1,056 us, 840 so).
 void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vector<BlendSpan>& spans,
                   double& model_makespan, std::vector<double>& item_work_out, bool sat = false) {
-    items.clear();
-    spans.clear();
-    std::vector<std::vector<double>> est(ctx->patches.size());
-    std::vector<int> tiles(ctx->patches.size());
+    const size_t np = ctx->patches.size();
+    std::vector<std::vector<double>> est(np);
+    std::vector<int> tiles(np);
     double total = 0.0;
-    for (size_t k = 0; k < ctx->patches.size(); ++k) {
+    for (size_t k = 0; k < np; ++k) {
         est[k] = sat ? tile_bucket_sat(*ctx->patches[k], tiles[k]) : tile_bucket_stages(*ctx->patches[k], tiles[k]);
         for (double e : est[k]) total += e;
-        total += kItemStages * tiles[k];
+        total += (sat ? kSatItemStages : kItemStages) * tiles[k];
     }
-    const double cap = 0.25 * total / std::max(slots, 1);
-    std::vector<double> work;
-    for (size_t k = 0; k < ctx->patches.size(); ++k) {
-        const PatchHost& P = *ctx->patches[k];
-        const int nb = P.T.nb, gmax = std::min(std::min(nb, 16), P.partial_planes);
-        int G = 1;
-        for (;; ++G) {
-            double mx = 0.0;
-            for (int t = 0; t < tiles[k]; ++t)
-                for (int g = 0; g < G; ++g) mx = std::max(mx, item_work(est[k], nb, t, g, G));
-            if (mx <= cap || G >= gmax) break;
-        }
-        // summed-area items: no more groups than the patch's own plan takes
-        // (enough waves for the patch alone; more only adds blend traffic),
-        // and each bucket's passes split over K parts where an item would
-        // still outlast the balanced per-slot share of the frame (dense
-        // patches whose buckets take many passes)
-        int K = 1;
-        if (sat) {
-            G = std::max(1, std::min(G, P.sat_groups));
-            double wmax = 0.0;
-            for (int t = 0; t < tiles[k]; ++t)
-                for (int g = 0; g < G; ++g) wmax = std::max(wmax, item_work(est[k], nb, t, g, G));
-            K = sat_parts_for(wmax, 4.0 * cap, std::max(1, std::min(8, P.partial_planes / G)));
-        }
+    const double per_slot = total / std::max(slots, 1);
+    auto group_work = [&](size_t k, int t, int g, int G) { return item_work(est[k], ctx->patches[k]->T.nb, t, g, G, sat); };
+    auto heaviest = [&](size_t k, int G) {
+        double mx = 0.0;
         for (int t = 0; t < tiles[k]; ++t)
-            for (int g = 0; g < G; ++g)
-                for (int q = 0; q < K; ++q) {
-                    items.push_back(K > 1 ? TcItem{P.index, t, g | (q << 16), G | (K << 16)} : TcItem{P.index, t, g, G});
-                    work.push_back(part_work(item_work(est[k], nb, t, g, G), K));
-                }
-        const std::vector<BlendSpan> sp = blend_spans(P, G * K);
-        spans.insert(spans.end(), sp.begin(), sp.end());
+            for (int g = 0; g < G; ++g) mx = std::max(mx, group_work(k, t, g, G));
+        return mx;
+    };
+    struct Plan {
+        std::vector<TcItem> items;
+        std::vector<BlendSpan> spans;
+        std::vector<double> work;
+        std::vector<int> order;
+        double makespan = 0.0, cost = 0.0;
+    } best;
+    const std::vector<double> shares = sat ? std::vector<double>{4.0, 2.0, 1.4, 1.0, 0.7, 0.5, 0.35, 0.25}
+                                           : std::vector<double>{0.25};
+    auto build = [&](double share, double gmul) {
+        const double cap = share * per_slot;
+        Plan pl;
+        double blend_us = 0.0;
+        for (size_t k = 0; k < np; ++k) {
+            const PatchHost& P = *ctx->patches[k];
+            const int nb = P.T.nb, gmax = std::min(std::min(nb, 16), P.partial_planes);
+            int G = 1;
+            while (G < gmax && heaviest(k, G) > cap) ++G;
+            G = std::max(1, std::min(gmax, (int)std::lround(G * gmul)));
+            // summed-area items: each bucket's passes split over K parts where
+            // an item would still outlast the balanced per-slot share of the
+            // frame (dense patches whose buckets take many passes)
+            int K = 1;
+            if (sat) K = sat_parts_for(heaviest(k, G), per_slot, std::max(1, std::min(8, P.partial_planes / G)));
+            for (int t = 0; t < tiles[k]; ++t)
+                for (int g = 0; g < G; ++g)
+                    for (int q = 0; q < K; ++q) {
+                        pl.items.push_back(K > 1 ? TcItem{P.index, t, g | (q << 16), G | (K << 16)}
+                                                 : TcItem{P.index, t, g, G});
+                        pl.work.push_back(part_work(group_work(k, t, g, G), K));
+                    }
+            const std::vector<BlendSpan> sp = blend_spans(P, G * K);
+            if (!sp.empty()) blend_us += (G * K + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs;
+            pl.spans.insert(pl.spans.end(), sp.begin(), sp.end());
+        }
+        pl.order.resize(pl.items.size());
+        for (size_t k = 0; k < pl.order.size(); ++k) pl.order[k] = (int)k;
+        std::stable_sort(pl.order.begin(), pl.order.end(), [&](int a, int b) { return pl.work[a] > pl.work[b]; });
+        pl.makespan = makespan(pl.work, pl.order, slots);
+        pl.cost = pl.makespan * kStageUs + blend_us + (pl.spans.empty() ? 0.0 : kBlendUs);
+        return pl;
+    };
+    double share = shares[0];
+    for (double c : shares) {
+        Plan pl = build(c, 1.0);
+        if (c == shares[0] || pl.cost < best.cost) {
+            std::swap(best, pl);
+            share = c;
+        }
     }
-    std::vector<int> order(items.size());
-    for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
-    model_makespan = makespan(work, order, slots);
-    std::vector<TcItem> sorted;
+    if (sat && ctx->sat_gmul != 1.0) best = build(share, ctx->sat_gmul);   // the autotuner's axis
+    model_makespan = best.makespan;
+    items.clear();
     item_work_out.clear();
-    for (int k : order) {
-        sorted.push_back(items[k]);
-        item_work_out.push_back(work[k]);
+    for (int k : best.order) {
+        items.push_back(best.items[k]);
+        item_work_out.push_back(best.work[k]);
     }
-    items.swap(sorted);
+    spans.swap(best.spans);
 }
 
 scwp_status ready(scwp_ctx* ctx) {
@@ -662,6 +690,13 @@ const PatchDev* patch_devs(scwp_ctx* ctx) {
     return ctx->devs.data();
 }
 
+// Whether the summed-area synthesis is one launch over all patches: in
+// batched mode, and for several patches always.  One launch per patch left
+// each to fill the chip alone, with as many bucket groups (partial planes, and
+// a blend pass of its own) as that takes: four patches of up to 500 cells a
+// side took 243 us a frame so, 160 with the frame's plan.
+bool one_synthesis(const scwp_ctx* ctx) { return ctx->batched || ctx->patches.size() > 1; }
+
 // device copies of the patch descriptors and synthesis parameters (and the
 // batched plan) after the set of patches or the batching mode changed
 scwp_status sync_synth(scwp_ctx* ctx) {
@@ -680,7 +715,7 @@ scwp_status sync_synth(scwp_ctx* ctx) {
     if (!ctx->d_pdevs || !ctx->d_sps) return fail(ctx, SCWP_E_NOMEM, "synthesis descriptors");
     CU(cudaMemcpyAsync(ctx->d_pdevs, pd.data(), n * sizeof(PatchDev), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(ctx->d_sps, sp.data(), n * sizeof(SynthParams), cudaMemcpyHostToDevice, ctx->st));
-    if (ctx->batched) {
+    if (one_synthesis(ctx)) {
         plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_makespan, ctx->b_work);
         ctx->d_bitems = (TcItem*)dalloc(ctx, std::max<size_t>(1, ctx->b_items.size()) * sizeof(TcItem));
         ctx->d_bspans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, ctx->b_spans.size()) * sizeof(BlendSpan));
@@ -715,7 +750,7 @@ scwp_status synthesize(scwp_ctx* ctx, int mode) {
             return ctx->sat_variant == 1 ? launch_synth_sat3(it, n, ctx->d_pdevs, ctx->d_sps, sp, ns, ctx->st)
                                          : launch_synth_sat(it, n, ctx->d_pdevs, ctx->d_sps, sp, ns, ctx->queue, ctx->st);
         };
-        if (ctx->batched) {
+        if (one_synthesis(ctx)) {
             CU(launch(ctx->d_sitems, (int)ctx->s_items.size(), ctx->d_sspans, (int)ctx->s_spans.size()));
         } else {
             for (PatchHost* P : ctx->patches)

@@ -44,12 +44,14 @@
 // them, in nearly every item; a bucket with more rows than the table spans
 // several segments, each a pass of its own).  Two batches are held: eight
 // warps build the next one (the next item's ticket, descriptors, bucket
-// geometry and row table: five dependent round trips to L2) in the y-prefix
+// geometry and row table: five dependent round trips to L2) in the x-prefix
 // phase of this one's last pass but one, which leaves them idle, so an item
-// starts without a wait and its first records are already on their way.
+// starts without a wait and its first records are already on their way
+// (512^2 patch, 100k particles: frame 144.7 -> 136.1 us).  One thread
+// describes the next pass in the y-prefix phase.
 // Within a pass each thread takes the candidates c0 + tid, c0 + tid + 1024,
-// ... on its own, with no barrier until the pass ends: it finds a
-// candidate's bin row (a binary search of the row table) and copies the
+// ... on its own, with no barrier until the pass ends: its warp finds the
+// candidates' bin rows (a ballot over the row table) and it copies the
 // record with asynchronous 16-byte copies (cp.async) into its own slot of
 // two, one candidate ahead, so the copy of its next candidate (of this pass,
 // or the first of the next pass) overlaps the current one's events, and the
@@ -58,13 +60,23 @@
 // candidate's support box to the tile and adds the nine weights at up to
 // four corners; bumps whose box starts at the tile's first texel in both axes
 // (every bump covering the whole tile among them) sum their (0, 0) corner in
-// registers, added by one warp reduction per pass.  Then the x prefix (one
-// row of one plane per thread), the y prefix (one column of one plane per
+// registers, added per lane to 32 words per plane that the x prefix sums.
+// Then the x prefix (one row of one plane per thread), the y prefix (one column of one plane per
 // thread, stored only at the first row of each 4-row segment of the
 // contraction) and the contraction (one column of a segment per thread),
 // which finishes the y prefix of the segment's other rows in registers and
 // zeroes every difference-array element it reads, so no pass needs a
 // clearing phase.
+//
+// What bounds it: shared-memory wavefronts and issue.  A pass of 1,000
+// candidates (1024^2 patch, 200k particles) takes about 13,000 cycles: events
+// 3,100 (75 a warp's 32 candidates), x prefix 3,250, y prefix 2,300,
+// contraction 3,100; the prefixes and the contraction alone are 6,048
+// wavefronts.  The description and the lane-wise corner took it from 16,000
+// (frame 311 -> 292 us; 8 patches of 2M particles 6.75 -> 6.45 ms).  Walking
+// quads of four columns along y with 144 threads, and scanning them along x
+// by shuffles in the contraction, was 15-20 % slower: too few warps to keep
+// the pipe busy, and as many wavefronts for the shuffles as they saved.
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
