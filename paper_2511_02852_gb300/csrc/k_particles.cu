@@ -138,21 +138,12 @@ __device__ __forceinline__ void clear_sort_words(const PatchDev& p) {
             p.sort_status[((size_t)ps * p.nblk_o + blockIdx.x) * 256 + threadIdx.x] = 0u;
 }
 
-// Particle i of the patch (where `ok`; every lane of the warp calls): its
-// crest's and trough's keys, its state packed for the record pass (one
-// 16-byte gather per bump instead of three 4-byte ones), its counts.
-__device__ __forceinline__ void add_keys(KeyCounts& C, const PatchDev& p, int i, int32_t x, int32_t y, uint32_t bd,
-                                         int4 vq, bool ok, unsigned long long& ev, unsigned int& binned) {
-    const int b = (int)(bd >> 16);
-    // live particles per bucket, one shared atomic per bucket and warp
-    // (neighbours mostly share theirs: one per particle met 32 ways in
-    // one word)
-    const uint32_t peers = __match_any_sync(0xffffffffu, ok ? b : -1);
-    if (!ok) return;
-    if ((peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicAdd(&C.live[b], (unsigned)__popc(peers));
-    p.pk[i] = make_int4(x, y, (int)bd, 0);
-    const BucketDev bk = p.bk[b];
-    uint32_t key[2];
+// The crest's and trough's keys of a particle (total_bins: the bump reaches
+// no texel) and its counts' share; whether either bump reaches the patch.
+__device__ __forceinline__ bool make_keys(const PatchDev& p, int32_t x, int32_t y, uint32_t bd, int4 vq,
+                                          uint32_t (&key)[2], unsigned long long& ev, unsigned int& binned) {
+    const BucketDev bk = p.bk[bd >> 16];
+    bool any = false;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int32_t cx = k ? x - vq.z : x;
@@ -167,9 +158,36 @@ __device__ __forceinline__ void add_keys(KeyCounts& C, const PatchDev& p, int i,
             key[k] = (uint32_t)(bk.base + by * bk.nbx + bx);
             ev += (unsigned long long)nx * (unsigned long long)ny;
             ++binned;
+            any = true;
         }
-        for (int ps = 0; ps < sort_passes(p); ++ps) atomicAdd(&C.h[ps][(key[k] >> (8 * ps)) & 255u], 1u);
     }
+    return any;
+}
+
+// A live particle's keys and bucket in the block's counts (where `ok`; every
+// lane of the warp calls).  Neighbours mostly share their bucket: one shared
+// atomic for such a warp (one per particle met 32 ways in one word).
+__device__ __forceinline__ void count_keys(KeyCounts& C, const PatchDev& p, uint32_t bd, const uint32_t (&key)[2],
+                                           bool ok) {
+    const unsigned act = __ballot_sync(0xffffffffu, ok);
+    if (act == 0u) return;
+    const uint32_t b = bd >> 16, b0 = __shfl_sync(0xffffffffu, b, __ffs(act) - 1);
+    const bool same = __all_sync(0xffffffffu, !ok || b == b0);
+    if (!ok) return;
+    if (!same)
+        atomicAdd(&C.live[b], 1u);
+    else if ((act & ((1u << (threadIdx.x & 31)) - 1u)) == 0u)
+        atomicAdd(&C.live[b], (unsigned)__popc(act));
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        for (int ps = 0; ps < sort_passes(p); ++ps) atomicAdd(&C.h[ps][(key[k] >> (8 * ps)) & 255u], 1u);
+}
+
+// Particle i's keys, and its state packed for the record pass (one 16-byte
+// gather per bump instead of three 4-byte ones).
+__device__ __forceinline__ void store_keys(const PatchDev& p, int i, int32_t x, int32_t y, uint32_t bd,
+                                           const uint32_t (&key)[2]) {
+    p.pk[i] = make_int4(x, y, (int)bd, 0);
     reinterpret_cast<uint2*>(p.keys[0])[i] = make_uint2(key[0], key[1]);
 }
 
@@ -247,23 +265,24 @@ __global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack
         xs[k] = i < n ? X[i] : 0;
         ys[k] = i < n ? Y[i] : 0;
     }
+    // a particle lives on while either of its bumps reaches the patch: the
+    // test that gives it its keys
     int4 vq[kItems];
-    uint32_t alive = 0u;
+    uint32_t alive = 0u, key[kItems][2];
+    unsigned long long ev = 0;
+    unsigned int binned = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) vq[k] = lookup_vq(p, bs[k]);
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
-        const int i = base + k * kTpb + tid;
-        const int32_t x = xs[k] + vq[k].x, y = ys[k] + vq[k].y;
-        xs[k] = x;
-        ys[k] = y;
-        const int32_t R = p.bk[bs[k] >> 16].R;
-        const bool a = i < n && ((span_count(x, R, p.W) > 0 && span_count(y, R, p.H) > 0) ||
-                                 (span_count(x - vq[k].z, R, p.W) > 0 && span_count(y - vq[k].w, R, p.H) > 0));
+        xs[k] += vq[k].x;
+        ys[k] += vq[k].y;
+        const bool a = base + k * kTpb + tid < n && make_keys(p, xs[k], ys[k], bs[k], vq[k], key[k], ev, binned);
         const uint32_t m = __ballot_sync(0xffffffffu, a);
         rank[k] = (uint32_t)__popc(m & ((1u << lane) - 1u));
         alive |= (a ? 1u : 0u) << k;
         if (lane == 0) s_cnt[k * (kTpb / 32) + warp] = (uint32_t)__popc(m);
+        count_keys(C, p, bs[k], key[k], a);
     }
     __syncthreads();
     if (warp == 0) {
@@ -311,18 +330,15 @@ __global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack
     int32_t* Xd = p.x[1 - p.cur];
     int32_t* Yd = p.y[1 - p.cur];
     uint32_t* Bd = p.bd[1 - p.cur];
-    unsigned long long ev = 0;
-    unsigned int binned = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
         const int o = (int)(s_off + s_cnt[k * (kTpb / 32) + warp] + rank[k]);
-        const bool a = (alive >> k) & 1u;
-        if (a) {
+        if ((alive >> k) & 1u) {
             Xd[o] = xs[k];
             Yd[o] = ys[k];
             Bd[o] = bs[k];
+            store_keys(p, o, xs[k], ys[k], bs[k], key[k]);
         }
-        add_keys(C, p, o, xs[k], ys[k], bs[k], vq[k], a, ev, binned);
     }
     keys_end(C, p, ev, binned);
 }
@@ -394,7 +410,12 @@ __device__ __forceinline__ void inject_body(const PatchDev& p, const IP& ip, con
             Y[idx] = y;
             BD[idx] = bd;
         }
-        add_keys(C, p, (int)idx, x, y, bd, ok ? lookup_vq(p, bd) : make_int4(0, 0, 0, 0), ok, ev, binned);
+        uint32_t key[2] = {0u, 0u};
+        if (ok) {
+            make_keys(p, x, y, bd, lookup_vq(p, bd), key, ev, binned);
+            store_keys(p, (int)idx, x, y, bd, key);
+        }
+        count_keys(C, p, bd, key, ok);
     }
     keys_end(C, p, ev, binned);
 }
@@ -479,7 +500,12 @@ __global__ void __launch_bounds__(kTpb) k_bin_keys(const __grid_constant__ Patch
 #pragma unroll
     for (int m = 0; m < kBinItems; ++m) {
         const int i = i0 + m * kTpb;
-        add_keys(C, p, i, px[m], py[m], bd[m], lookup_vq(p, bd[m]), i < n, ev, binned);
+        uint32_t key[2] = {0u, 0u};
+        if (i < n) {
+            make_keys(p, px[m], py[m], bd[m], lookup_vq(p, bd[m]), key, ev, binned);
+            store_keys(p, i, px[m], py[m], bd[m], key);
+        }
+        count_keys(C, p, bd[m], key, i < n);
     }
     keys_end(C, p, ev, binned);
 }
