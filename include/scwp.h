@@ -298,6 +298,15 @@ scwp_status scwp_get_bins(scwp_ctx* ctx, int32_t patch_id, uint32_t* counts, uin
  * CUDA context and every other scwp context stay usable.  Synchronises. */
 scwp_status scwp_debug_sort_timeout(scwp_ctx* ctx, int32_t patch_id, double wait_seconds);
 
+/* The same self-test of the step kernel's look-back: the step of the patch's
+ * live particles with the word of its first tile of 1024 particles never
+ * published, then the frame's binning, which must take the patch as empty (as
+ * every stage does after a wait that timed out).  Needs at least 1025 live
+ * particles (two tiles), else SCWP_E_INVALID.  Returns SCWP_E_TIMEOUT (sticky)
+ * when the kernel reported the timeout and no bump was binned after it,
+ * SCWP_E_STATE otherwise.  Synchronises. */
+scwp_status scwp_debug_step_timeout(scwp_ctx* ctx, int32_t patch_id, double wait_seconds);
+
 /* Recompute the synthesis and blend of every patch from the current
  * particles and background without advancing the frame (the bins are
  * rebuilt).  mode: any SCWP_SYNTH_* (SCWP_SYNTH_SAT, the default path of

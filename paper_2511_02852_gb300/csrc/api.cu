@@ -1936,21 +1936,52 @@ scwp_status scwp_get_bins(scwp_ctx* ctx, int32_t patch_id, uint32_t* counts, uin
     return SCWP_OK;
 }
 
-scwp_status scwp_debug_sort_timeout(scwp_ctx* ctx, int32_t patch_id, double wait_seconds) {
+// Arguments of a look-back self-test on a patch, and its limit in SM clocks.
+static scwp_status stall_args(scwp_ctx* ctx, int32_t patch_id, double wait_seconds, int32_t& live, long long& cycles) {
     scwp_status s = ready(ctx);
     if (s != SCWP_OK) return s;
     if (patch_id < 0 || patch_id >= (int)ctx->patches.size() || !(wait_seconds > 0.0) || wait_seconds > 2.0)
         return fail(ctx, SCWP_E_INVALID, "args");
-    PatchHost* P = ctx->patches[patch_id];
-    int32_t cnt = 0;
-    CU(cudaMemcpyAsync(&cnt, P->dev.count, sizeof(cnt), cudaMemcpyDeviceToHost, ctx->st));
+    CU(cudaMemcpyAsync(&live, ctx->patches[patch_id]->dev.count, sizeof(live), cudaMemcpyDeviceToHost, ctx->st));
     CU(cudaStreamSynchronize(ctx->st));
-    // at least two sort tiles of bump keys: tile 1 then looks back to tile 0
-    if (2 * (int64_t)cnt <= kSortPassTile) return fail(ctx, SCWP_E_INVALID, "too few particles for two sort tiles");
     int dev = 0, khz = 0;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev));
-    const long long cycles = (long long)(wait_seconds * 1e3 * (double)(khz > 0 ? khz : 2070000));
+    cycles = (long long)(wait_seconds * 1e3 * (double)(khz > 0 ? khz : 2070000));
+    return SCWP_OK;
+}
+
+scwp_status scwp_debug_step_timeout(scwp_ctx* ctx, int32_t patch_id, double wait_seconds) {
+    int32_t live = 0;
+    long long cycles = 0;
+    scwp_status s = stall_args(ctx, patch_id, wait_seconds, live, cycles);
+    if (s != SCWP_OK) return s;
+    // at least two step tiles: tile 1 then looks back to tile 0
+    if (live <= kStepTile) return fail(ctx, SCWP_E_INVALID, "too few particles for two step tiles");
+    PatchDev& D = ctx->patches[patch_id]->dev;
+    graph_reset(ctx);
+    CU(launch_step_stall(D, cycles, ctx->st));
+    D.cur ^= 1;
+    CU(launch_bin(&D, 1, false, ctx->st));
+    unsigned long long flags = 0;
+    std::vector<uint32_t> off((size_t)D.total_bins + 1);
+    CU(cudaMemcpyAsync(&flags, D.stats + 2, sizeof(flags), cudaMemcpyDeviceToHost, ctx->st));
+    CU(cudaMemcpyAsync(off.data(), D.offsets, off.size() * 4, cudaMemcpyDeviceToHost, ctx->st));
+    CU(cudaStreamSynchronize(ctx->st));
+    if (!(flags & kErrTimeout)) return fail(ctx, SCWP_E_STATE, "the step look-back self-test did not time out");
+    for (uint32_t o : off)
+        if (o != 0) return fail(ctx, SCWP_E_STATE, "bumps binned after the step's look-back timed out");
+    return fail(ctx, SCWP_E_TIMEOUT, "a device wait timed out (step look-back self-test)");
+}
+
+scwp_status scwp_debug_sort_timeout(scwp_ctx* ctx, int32_t patch_id, double wait_seconds) {
+    int32_t live = 0;
+    long long cycles = 0;
+    scwp_status s = stall_args(ctx, patch_id, wait_seconds, live, cycles);
+    if (s != SCWP_OK) return s;
+    // at least two sort tiles of bump keys: tile 1 then looks back to tile 0
+    if (2 * (int64_t)live <= kSortPassTile) return fail(ctx, SCWP_E_INVALID, "too few particles for two sort tiles");
+    PatchHost* P = ctx->patches[patch_id];
     graph_reset(ctx);
     CU(launch_sort_stall(P->dev, cycles, ctx->st));
     unsigned long long flags = 0;

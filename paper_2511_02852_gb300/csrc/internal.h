@@ -234,6 +234,9 @@ cudaError_t launch_bin(const PatchDev* ps, int n, bool keys, cudaStream_t st);
 // its first tile never taken, so the look-back waits on it give up after
 // wait_cycles SM clocks and set the timeout flag (outputs meaningless)
 cudaError_t launch_sort_stall(const PatchDev& p, long long wait_cycles, cudaStream_t st);
+// the same of the step's look-back (the caller flips `cur` after it; the
+// frame's binning then takes the patch as empty)
+cudaError_t launch_step_stall(const PatchDev& p, long long wait_cycles, cudaStream_t st);
 cudaError_t launch_synth_gather(const PatchDev& p, const SynthParams& sp, cudaStream_t st);
 // Tensor-core synthesis of `n_items` items (any patches) in one launch, then
 // the group-sum blend of `n_spans` spans in one launch.  `pdevs` and `sps`

@@ -113,6 +113,20 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* a) {
     return v;
 }
 
+// The live particles a patch's kernels take: none once one of its bounded waits
+// has run out.  A step or a sort pass that gave up leaves counts, digit totals
+// and keys that no longer agree; a later pass that trusted them would store
+// past the key buffers, the records would be gathered by ids from places that
+// nothing wrote, and the synthesis would follow bin offsets that run backwards.
+// From the kernel after the one that gave up on, the patch is empty instead:
+// no keys, every bin offset zero.  A kernel with such waits reads the count in
+// one thread for its block, as the flag may be set while it runs.
+__device__ __forceinline__ int live_count(const PatchDev& p) {
+    const unsigned long long err = p.stats[2];
+    const int n = p.count[0];   // (both loads in flight together)
+    return (err & kErrTimeout) ? 0 : n;
+}
+
 // ---- a6: bin keys -------------------------------------------------------------
 // A block's counts while it makes keys: every sort pass's digits (so the
 // passes need no histogram launch), live particles per bucket, evaluations
@@ -230,26 +244,36 @@ __device__ __forceinline__ void keys_end(KeyCounts& C, const PatchDev& p, unsign
 // written and read back twice) and took three of a small frame's nine serial
 // launches; this moves 48 and is one.  The tile of the last particle
 // publishes the new count: by then every block with a tile has read the old
-// one, since that tile has seen all their counts.
+// one, since that tile has seen all their counts.  A tile that gives up on its
+// look-back (after wait_cycles SM clocks) sets the error flag and has summed a
+// subset of the earlier tiles' counts: its stores stay in bounds, and the
+// stages after it take the patch as empty (live_count).  Tickets start at tile
+// first_tile: 0 in every frame, 1 in the failure-detection self-test, whose
+// tile 0 nothing publishes.
 template <int M>
-__global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack<M> pk) {
+__global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack<M> pk, long long wait_cycles,
+                                               int first_tile) {
     __shared__ KeyCounts C;
     __shared__ uint32_t s_cnt[32], s_off;   // survivors of 32-particle runs, then the runs' offsets
-    __shared__ int s_bid;
+    __shared__ int s_bid, s_n;
     static_assert(kItems * kTpb / 32 == 32, "one run per lane of the scanning warp");
     const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
     if (M > 1 && (int)blockIdx.x >= p.nblk_c) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t* const words = p.blk;          // [nblk_c] look-back words, then the ticket
-    if (tid == 0) s_bid = (int)atomicAdd(words + p.nblk_c, 1u);
+    if (tid == 0) {
+        const int t = (int)atomicAdd(words + p.nblk_c, 1u);   // (in flight beside the count)
+        s_n = live_count(p);
+        s_bid = t + first_tile;
+    }
     clear_sort_words(p);
     keys_begin(C, p);
     __syncthreads();
     const int bid = s_bid;
-    const int n = p.count[0], base = bid * kTileC;
+    const int n = s_n, base = bid * kTileC;
     if (base >= n) {   // (uniform)
-        if (n == 0 && bid == 0 && tid == 0) p.count[1] = 0;
+        if (n == 0 && bid == 0 && tid == 0) p.count[0] = p.count[1] = 0;
         return;
     }
     const int32_t* X = p.x[p.cur];
@@ -312,7 +336,7 @@ __global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack
                 if (done) break;
                 j -= fu;
                 bool late = false;
-                if (lane == 0 && fu < 32) late = clock64() - t0 > kLbWaitCycles;
+                if (lane == 0 && fu < 32) late = clock64() - t0 > wait_cycles;
                 if (__any_sync(0xffffffffu, late)) {
                     // (excl is then below the true offset: every store stays in bounds)
                     if (lane == 0) atomicOr(&p.stats[2], (unsigned long long)kErrTimeout);
@@ -475,7 +499,7 @@ __global__ void __launch_bounds__(kTpb) k_bin_keys(const __grid_constant__ Patch
     pdl_enter();
     if (M > 1 && (int)blockIdx.x >= p.nblk_s) return;
     clear_sort_words(p);
-    const int n = p.count[0];
+    const int n = live_count(p);
     const int32_t* X = p.x[p.cur];
     const int32_t* Y = p.y[p.cur];
     const uint32_t* BD = p.bd[p.cur];
@@ -573,7 +597,7 @@ __global__ void __launch_bounds__(kSortTpb, 3) k_sort_pass(const __grid_constant
     __shared__ uint32_t s_ls[256];              // the digit's first position in the reordered tile
     __shared__ uint32_t s_gb[256];              // output position of reordered tile position 0 of the digit
     __shared__ uint32_t s_warp[8];
-    __shared__ int s_bid;
+    __shared__ int s_bid, s_n;
     __shared__ bool s_last;
     const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
@@ -588,8 +612,10 @@ __global__ void __launch_bounds__(kSortTpb, 3) k_sort_pass(const __grid_constant
     uint32_t* const ticket = p.sort_ticket + 2 * ps;
     unsigned long long* const err = p.stats + 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = 2 * p.count[0];
-    const uint32_t gd = block_exscan256(tid < 256 ? dtot[tid] : 0u, s_warp);   // keys of smaller digits, all tiles
+    const uint32_t dt = tid < 256 ? dtot[tid] : 0u;
+    if (tid == 0) s_n = 2 * live_count(p);   // (read after the scan's barrier)
+    const uint32_t gd = block_exscan256(dt, s_warp);   // keys of smaller digits, all tiles
+    const int n = s_n;
     const uint32_t lt = (1u << lane) - 1u;
     for (;;) {
         if (tid == 0) s_bid = (int)atomicAdd(ticket, 1u) + first_tile;
@@ -749,6 +775,7 @@ __global__ void __launch_bounds__(kTpb) k_offsets_records(const __grid_constant_
     __shared__ uint4 s_rec[kTpb / 32][64];
     const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
+    const int n = 2 * live_count(p);
     const uint32_t* const keys = p.keys[sort_passes(p) & 1];
     const uint32_t* const vals = p.vals[sort_passes(p) & 1];
     // the frame's statistics (the error flags stay; the synthesis counts its
@@ -769,7 +796,6 @@ __global__ void __launch_bounds__(kTpb) k_offsets_records(const __grid_constant_
         if (t == p.nb) p.stats[3 + p.nb] = p.stats[5 + p.nb] = 0ull;
     }
     for (int i = blockIdx.x * kTpb + threadIdx.x; i <= p.nblk_c; i += gridDim.x * kTpb) p.blk[i] = 0u;
-    const int n = 2 * p.count[0];
     const int4* PK = p.pk;
     const uint32_t tb = (uint32_t)p.total_bins;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -892,7 +918,7 @@ cudaError_t launch_step(const PatchDev* ps, int n, cudaStream_t st) {
         constexpr int M = std::decay_t<decltype(pk)>::kM;
         count_launches(1);
         return launch_pdl(k_step<M>, dim3(pack_max(pk, m, [](const PatchDev& p) { return p.nblk_c; }), m), kTpb, 0, st,
-                          pk);
+                          pk, kLbWaitCycles, 0);
     });
 }
 
@@ -964,6 +990,13 @@ cudaError_t launch_bin(const PatchDev* ps, int n, bool keys, cudaStream_t st) {
         count_launches(1);
         return launch_pdl(k_offsets_records<M>, dim3(std::min(rb, std::max(1, sm_count()) * 8), m), kTpb, 0, st, pk);
     });
+}
+
+cudaError_t launch_step_stall(const PatchDev& p, long long wait_cycles, cudaStream_t st) {
+    PatchPack<1> pk;
+    pk.p[0] = p;
+    count_launches(1);
+    return launch_pdl(k_step<1>, dim3(p.nblk_c), kTpb, 0, st, pk, wait_cycles, 1);
 }
 
 int sorted_buffer_index(const PatchDev& p) { return sort_passes(p) & 1; }
