@@ -99,6 +99,10 @@ struct scwp_ctx {
     int device = -1;                  // the device the context was made on
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    // a server's scene: its last asynchronous read of the background on st,
+    // which the next background, made on another stream, must wait for
+    cudaEvent_t ev_bg_read = nullptr;
+    bool bg_read = false;
     std::string err;
     scwp_status sticky = SCWP_OK;
     SpectrumModel sm;
@@ -1666,6 +1670,21 @@ static cudaError_t copy_map(scwp_ctx* ctx, float* dst, const float* src, size_t 
     return cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToDevice, ctx->st);
 }
 
+// After an asynchronous read of the background on the context's stream.  A
+// context of its own makes its next background behind that stream; a server's
+// ticks make theirs on a stream that waits for this event.  (A read captured
+// into a graph leaves nothing to wait for here: the graph's owner orders its
+// replays.)
+static scwp_status background_read(scwp_ctx* ctx) {
+    if (!ctx->ev_bg_read) return SCWP_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing(ctx->st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return SCWP_OK;
+    CU(cudaEventRecord(ctx->ev_bg_read, ctx->st));
+    ctx->bg_read = true;
+    return SCWP_OK;
+}
+
 scwp_status scwp_height_map(scwp_ctx* ctx, int32_t patch_id, int32_t field, float* dst, size_t dst_elems,
                             int32_t dst_on_device) {
     scwp_status s = ready(ctx);
@@ -1685,6 +1704,7 @@ scwp_status scwp_height_map(scwp_ctx* ctx, int32_t patch_id, int32_t field, floa
     if (dst_elems < n) return fail(ctx, SCWP_E_INVALID, "dst too small");
     if (dst_on_device) {
         CU(copy_map(ctx, dst, src, n));
+        if (patch_id == -1 && (s = background_read(ctx)) != SCWP_OK) return s;
     } else {
         CU(cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToHost, ctx->st));
         CU(cudaStreamSynchronize(ctx->st));
@@ -1710,6 +1730,7 @@ scwp_status scwp_height_maps(scwp_ctx* ctx, int32_t patch_id, float* dst, size_t
     if (dst_elems < 3 * n) return fail(ctx, SCWP_E_INVALID, "dst too small");
     if (dst_on_device) {
         CU(copy_map(ctx, dst, src, 3 * n));
+        if (patch_id == -1 && (s = background_read(ctx)) != SCWP_OK) return s;
     } else {
         CU(cudaMemcpyAsync(dst, src, 3 * n * sizeof(float), cudaMemcpyDeviceToHost, ctx->st));
         CU(cudaStreamSynchronize(ctx->st));
@@ -2037,6 +2058,7 @@ void scwp_destroy(scwp_ctx* ctx) {
     dfree_all(ctx);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    if (ctx->ev_bg_read) cudaEventDestroy(ctx->ev_bg_read);
     if (ctx->side) cudaStreamDestroy(ctx->side);
     cudaGetLastError();
     delete ctx;
@@ -2171,6 +2193,12 @@ scwp_status scwp_server_add_scene(scwp_server* sv, const scwp_spectrum_desc* spe
     scwp_ctx* ctx = nullptr;
     scwp_status s = scwp_create(&d, &ctx);
     if (s != SCWP_OK) return sfail(sv, s, "scene: scwp_create failed");
+    if (cudaEventCreateWithFlags(&ctx->ev_bg_read, cudaEventDisableTiming) != cudaSuccess) {
+        ctx->ev_bg_read = nullptr;
+        cudaGetLastError();
+        scwp_destroy(ctx);
+        return sfail(sv, SCWP_E_CUDA, "scene: event");
+    }
     for (int32_t k = 0; k < n_patches && s == SCWP_OK; ++k) {
         int32_t pid = 0;
         s = scwp_add_patch(ctx, patches + k, &pid);
@@ -2330,7 +2358,14 @@ scwp_status scwp_server_tick(scwp_server* sv, int32_t* started) {
     memcpy(h + o_ip, ips.data(), ips.size() * sizeof(InjectParams));
     unsigned char* dv = (unsigned char*)sv->dstage[slot];
     // the backgrounds, then the particle stages of every patch, beside each
-    // other on the tick streams; the synthesis waits for both
+    // other on the tick streams; the synthesis waits for both.  A background
+    // that a caller's copy on the server stream has yet to read waits for it
+    // (the patch maps are written on that stream, behind any such copy).
+    for (int i : take) {
+        scwp_ctx* c = sv->scenes[i].ctx;
+        if (c->bg_read) SCU(cudaStreamWaitEvent(sv->pst[1], c->ev_bg_read, 0));
+        c->bg_read = false;
+    }
     SCU(launch_backgrounds(bgs.data(), bg_t.data(), (int)bgs.size(), sv->pst[1]));
     SCU(cudaMemcpyAsync(dv, h, bytes, cudaMemcpyHostToDevice, sv->pst[0]));
     const int np = (int)pd.size();
