@@ -3,6 +3,7 @@
 // the copy / inspection calls.  Host bookkeeping that decides integers (the
 // injection carries, the wake's quantised angle) is float64 and lives in
 // host_spectrum.cpp / here, compiled without floating-point contraction.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -1651,20 +1652,36 @@ scwp_status scwp_autotune(scwp_ctx* ctx, int32_t reps, int32_t force, scwp_tune_
     return SCWP_OK;
 }
 
-// A map to the caller's device buffer: by a kernel where the buffer lies on
-// this context's device and that device is current, else (another device's
-// memory, managed or mapped memory, anything that is no device allocation) by
-// the copy API, which takes or refuses it.
+// Whether [q, q + bytes) lies in one device allocation.
+static bool in_one_allocation(const void* q, size_t bytes) {
+    using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const RangeFn range = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) !=
+                cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<RangeFn>(fn);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr d = (CUdeviceptr)(uintptr_t)q;
+    return range && range(&base, &size, d) == CUDA_SUCCESS && d >= base && bytes <= size && d - base <= size - bytes;
+}
+
+// A map to the caller's device buffer: by a kernel where the whole buffer lies
+// in one allocation on this context's device and that device is current, else
+// (another device's memory, managed or mapped memory, anything that is no
+// device allocation or reaches past one) by the copy API, which takes or
+// refuses it.
 static cudaError_t copy_map(scwp_ctx* ctx, float* dst, const float* src, size_t n) {
     int dev = -1;
     if (cudaGetDevice(&dev) == cudaSuccess && dev == ctx->device && ((uintptr_t)dst & 3u) == 0) {
-        bool here = true;
-        for (const float* q : {dst, dst + n - 1}) {
-            cudaPointerAttributes a{};
-            here = here && cudaPointerGetAttributes(&a, q) == cudaSuccess && a.type == cudaMemoryTypeDevice &&
-                   a.device == dev;
-        }
-        if (here) return launch_copy(src, dst, n, ctx->st);
+        cudaPointerAttributes a{};
+        if (cudaPointerGetAttributes(&a, dst) == cudaSuccess && a.type == cudaMemoryTypeDevice && a.device == dev &&
+            in_one_allocation(dst, n * sizeof(float)))
+            return launch_copy(src, dst, n, ctx->st);
     }
     cudaGetLastError();
     return cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToDevice, ctx->st);
