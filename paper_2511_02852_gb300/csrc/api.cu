@@ -12,10 +12,8 @@
 #include <algorithm>
 #include <deque>
 #include <cmath>
-#include <functional>
 #include <map>
 #include <mutex>
-#include <queue>
 #include <new>
 #include <string>
 #include <vector>
@@ -146,9 +144,7 @@ struct scwp_ctx {
     std::vector<BlendSpan> s_spans;
     TcItem* d_sitems = nullptr;
     BlendSpan* d_sspans = nullptr;
-    double s_makespan = 0.0;
     std::vector<double> s_work;
-    double b_makespan = 0.0;
     // captured batched frames (one per parity of the particle buffers)
     FrameGraph gfull;                 // whole batched frames (scwp_step)
     cudaStream_t gst = nullptr;       // capture origin (the caller's stream may be the legacy one)
@@ -339,40 +335,98 @@ constexpr double kItemStages = 2.0;   // set-up and read-out of one item, in sta
 constexpr double kStageUs = 1.3;      // one stage on one CTA slot (two CTAs per SM)
 constexpr double kHbmBytesPerUs = 6.8e6;
 
-// expected operand stages of every (tile, bucket) of a patch, [tiles][nb]
-std::vector<double> tile_bucket_stages(const PatchHost& P, int& tiles) {
+// Estimated work of a patch's (tile, bucket) pairs.  Tiles of the same
+// estimates share a class: a plan weighs each class once, whatever the number
+// of its tiles.
+struct TileWork {
+    int tiles = 0, nb = 0;
+    std::vector<double> est;              // [classes][nb]
+    std::vector<std::vector<int>> cls;    // the classes' tiles, ascending
+};
+
+// The classes of a patch's tiles: of each column (row) k a signature
+// sig(k, bucket), equal signatures one class of columns (rows); a tile's class
+// is its column's and row's.  rep: a column and row of each class.
+template <typename SX, typename SY>
+void tile_classes(TileWork& tw, int ntx, int nty, int nb, SX&& sx, SY&& sy, std::vector<std::pair<int, int>>& rep) {
+    auto axis = [nb](int n, auto&& sig, std::vector<int>& first, std::vector<int>& of) {
+        for (int k = 0; k < n; ++k) {
+            size_t j = 0;
+            for (; j < first.size(); ++j) {
+                int i = 0;
+                while (i < nb && sig(k, i) == sig(first[j], i)) ++i;
+                if (i == nb) break;
+            }
+            if (j == first.size()) first.push_back(k);
+            of.push_back((int)j);
+        }
+    };
+    std::vector<int> fx, fy, cx, cy;
+    axis(ntx, sx, fx, cx);
+    axis(nty, sy, fy, cy);
+    tw.tiles = ntx * nty;
+    tw.nb = nb;
+    tw.cls.resize(fx.size() * fy.size());
+    for (int t = 0; t < tw.tiles; ++t) tw.cls[(size_t)cy[t / ntx] * fx.size() + cx[t % ntx]].push_back(t);
+    tw.est.resize(tw.cls.size() * nb);
+    for (int y : fy)
+        for (int x : fx) rep.push_back({x, y});
+}
+
+// expected bumps of a patch per bucket and texel of the bucket's domain
+std::vector<double> bump_density(const PatchHost& P) {
     const PatchTablesHost& T = P.T;
-    const int ts = synth_tc_tile(), kc = synth_tc_stage_bumps();
-    const int ntx = (T.W + ts - 1) / ts, nty = (T.H + ts - 1) / ts;
-    tiles = ntx * nty;
     // bumps: two per live particle (crest and trough)
     const double total = 2.0 * (P.d.prefill > 0 ? (double)P.d.prefill : 0.5 * (double)P.d.max_particles);
-    std::vector<double> w(T.nb);
+    std::vector<double> w(T.nb), dens(T.nb);
     double sw = 0.0;
     for (int i = 0; i < T.nb; ++i) {
         w[i] = ((double)T.W * kQ + 2.0 * T.R[i]) / ((double)T.R[i] * (double)T.R[i]);
         sw += w[i];
     }
-    std::vector<double> est((size_t)tiles * T.nb);
     for (int i = 0; i < T.nb; ++i) {
         const double r = (double)T.R[i] / kQ;
-        const double dens = total * w[i] / sw / ((T.W + 2 * r) * (T.H + 2 * r));
-        for (int t = 0; t < tiles; ++t) {
-            const double x0 = (t % ntx) * ts - r, x1 = (t % ntx + 1) * ts + r;
-            const double y0 = (t / ntx) * ts - r, y1 = (t / ntx + 1) * ts + r;
-            const double ax = std::max(0.0, std::min(x1, T.W + r) - std::max(x0, -r));
-            const double ay = std::max(0.0, std::min(y1, T.H + r) - std::max(y0, -r));
-            // bump centres that cover the whole tile go through the 3 x 3
-            // moments, not the MMAs: the box (x_last - r, x_first + r),
-            // shrunk by half a bin on each side for the bin rounding
-            // (x0, x1 are the tile grown by r: the box is (x1 - 2r, x0 + 2r))
-            const double hc = 0.5 * P.bin_cells[i];
-            const double fx = std::max(0.0, std::min(x0 + 2 * r - hc, T.W + r) - std::max(x1 - 2 * r + hc, -r));
-            const double fy = std::max(0.0, std::min(y0 + 2 * r - hc, T.H + r) - std::max(y1 - 2 * r + hc, -r));
-            est[(size_t)t * T.nb + i] = std::ceil(dens * std::max(0.0, ax * ay - fx * fy) / kc);
-        }
+        dens[i] = total * w[i] / sw / ((T.W + 2 * r) * (T.H + 2 * r));
     }
-    return est;
+    return dens;
+}
+
+// expected operand stages of every (tile, bucket) of a patch
+TileWork tile_bucket_stages(const PatchHost& P) {
+    const PatchTablesHost& T = P.T;
+    const int ts = synth_tc_tile(), kc = synth_tc_stage_bumps();
+    const int ntx = (T.W + ts - 1) / ts, nty = (T.H + ts - 1) / ts, nb = T.nb;
+    const std::vector<double> dens = bump_density(P);
+    // per bucket and column (row): the tile's reach inside the particle
+    // domain, and the bump centres that cover the whole tile.  Those go
+    // through the 3 x 3 moments, not the MMAs: the box (x_last - r, x_first +
+    // r), shrunk by half a bin on each side for the bin rounding (x0, x1 are
+    // the tile grown by r: the box is (x1 - 2r, x0 + 2r))
+    auto reach = [&](int n, int len, std::vector<std::pair<double, double>>& v) {
+        v.resize((size_t)n * nb);
+        for (int k = 0; k < n; ++k)
+            for (int i = 0; i < nb; ++i) {
+                const double r = (double)T.R[i] / kQ, hc = 0.5 * P.bin_cells[i];
+                const double x0 = k * ts - r, x1 = (k + 1) * ts + r;
+                v[(size_t)k * nb + i] = {
+                    std::max(0.0, std::min(x1, len + r) - std::max(x0, -r)),
+                    std::max(0.0, std::min(x0 + 2 * r - hc, len + r) - std::max(x1 - 2 * r + hc, -r))};
+            }
+    };
+    std::vector<std::pair<double, double>> rx, ry;
+    reach(ntx, T.W, rx);
+    reach(nty, T.H, ry);
+    TileWork out;
+    std::vector<std::pair<int, int>> rep;
+    tile_classes(out, ntx, nty, nb, [&](int k, int i) { return rx[(size_t)k * nb + i]; },
+                 [&](int k, int i) { return ry[(size_t)k * nb + i]; }, rep);
+    for (size_t c = 0; c < rep.size(); ++c)
+        for (int i = 0; i < nb; ++i) {
+            const auto& x = rx[(size_t)rep[c].first * nb + i];
+            const auto& y = ry[(size_t)rep[c].second * nb + i];
+            out.est[c * nb + i] = std::ceil(dens[i] * std::max(0.0, x.first * y.first - x.second * y.second) / kc);
+        }
+    return out;
 }
 
 // Work of the summed-area synthesis per (tile, bucket), in the same stage
@@ -387,55 +441,49 @@ constexpr double kSatItemStages = 2.0;
 constexpr double kBlendUs = 3.0;
 constexpr double kBlendBytesPerUs = 6.0e6;
 
-std::vector<double> tile_bucket_sat(const PatchHost& P, int& tiles, double* max_passes = nullptr) {
+// A tile's estimates depend on its column and row only through how far its
+// reach (grown by a bin) runs before the patch's domain ends: the tiles away
+// from the last columns and rows are one class.  (All terms are multiples of
+// 2^-16 far below 2^37: the differences are exact in float64.)
+TileWork tile_bucket_sat(const PatchHost& P, double* max_passes = nullptr) {
     const PatchTablesHost& T = P.T;
     const int ts = synth_sat_tile();
-    const int ntx = (T.W + ts - 1) / ts, nty = (T.H + ts - 1) / ts;
-    tiles = ntx * nty;
-    const double total = 2.0 * (P.d.prefill > 0 ? (double)P.d.prefill : 0.5 * (double)P.d.max_particles);
-    std::vector<double> w(T.nb);
-    double sw = 0.0;
-    for (int i = 0; i < T.nb; ++i) {
-        w[i] = ((double)T.W * kQ + 2.0 * T.R[i]) / ((double)T.R[i] * (double)T.R[i]);
-        sw += w[i];
-    }
-    std::vector<double> est((size_t)tiles * T.nb);
-    for (int i = 0; i < T.nb; ++i) {
-        const double r = (double)T.R[i] / kQ, c = (double)P.bin_cells[i];
-        const double dens = total * w[i] / sw / ((T.W + 2 * r) * (T.H + 2 * r));
-        for (int t = 0; t < tiles; ++t) {
-            const double x0 = (t % ntx) * ts - r, x1 = (t % ntx + 1) * ts + r;
-            const double y0 = (t / ntx) * ts - r, y1 = (t / ntx + 1) * ts + r;
-            const double ax = std::max(0.0, std::min(x1 + c, T.W + r) - std::max(x0, -r));
-            const double ay = std::max(0.0, std::min(y1 + c, T.H + r) - std::max(y0, -r));
+    const int ntx = (T.W + ts - 1) / ts, nty = (T.H + ts - 1) / ts, nb = T.nb;
+    const std::vector<double> dens = bump_density(P);
+    // extent of tile k's reach along an axis of `len` texels, without the bucket's 2 r
+    auto extent = [&](int k, int len, int i) {
+        return std::min((k + 1.0) * ts + P.bin_cells[i], (double)len) - (double)k * ts;
+    };
+    TileWork out;
+    std::vector<std::pair<int, int>> rep;
+    tile_classes(out, ntx, nty, nb, [&](int k, int i) { return extent(k, T.W, i); },
+                 [&](int k, int i) { return extent(k, T.H, i); }, rep);
+    for (size_t c = 0; c < rep.size(); ++c)
+        for (int i = 0; i < nb; ++i) {
+            const double r = (double)T.R[i] / kQ;
+            const double ax = extent(rep[c].first, T.W, i) + 2 * r, ay = extent(rep[c].second, T.H, i) + 2 * r;
             // dense pairs go in several passes, each with the fixed part
-            const double n = dens * ax * ay;
+            const double n = dens[i] * ax * ay;
             const double passes = std::max(1.0, std::ceil(n * std::sqrt(n) / (double)P.bk[i].sat_c));
             if (max_passes) *max_passes = std::max(*max_passes, passes);
-            est[(size_t)t * T.nb + i] = (passes * kSatBucketUs + n * kSatBumpUs) / kStageUs;
+            out.est[c * nb + i] = (passes * kSatBucketUs + n * kSatBumpUs) / kStageUs;
         }
-    }
-    return est;
+    return out;
 }
 
-double item_work(const std::vector<double>& est, int nb, int t, int g, int G, bool sat = false) {
+// work of the item of group g of G over a tile of class c
+double item_work(const TileWork& tw, size_t c, int g, int G, bool sat = false) {
     double s = sat ? kSatItemStages : kItemStages;
-    for (int i = (g * nb) / G; i < ((g + 1) * nb) / G; ++i) s += est[(size_t)t * nb + i];
+    for (int i = (g * tw.nb) / G; i < ((g + 1) * tw.nb) / G; ++i) s += tw.est[c * tw.nb + i];
     return s;
 }
 
-// makespan of in-order dispatch of `work` (already in launch order) on `slots`
-double makespan(const std::vector<double>& work, const std::vector<int>& order, int slots) {
-    std::priority_queue<double, std::vector<double>, std::greater<double>> q;
-    for (int k = 0; k < std::max(slots, 1); ++k) q.push(0.0);
-    double m = 0.0;
-    for (int it : order) {
-        const double f = q.top() + work[it];
-        q.pop();
-        q.push(f);
-        m = std::max(m, f);
-    }
-    return m;
+// the heaviest item of a patch in G groups
+double heaviest_item(const TileWork& tw, int G, bool sat = false) {
+    double mx = 0.0;
+    for (size_t c = 0; c < tw.cls.size(); ++c)
+        for (int g = 0; g < G; ++g) mx = std::max(mx, item_work(tw, c, g, G, sat));
+    return mx;
 }
 
 std::vector<BlendSpan> blend_spans(const PatchHost& P, int G) {
@@ -457,75 +505,134 @@ int sat_parts_for(double wmax, double cap, int kmax) {
 }
 double part_work(double w, int K) { return K > 1 ? kSatItemStages + (w - kSatItemStages) / K : w; }
 
+// The items of one launch, heaviest first, as runs of equal work: the tiles
+// of a class in one group (each in K parts).
+struct ItemRuns {
+    struct Run {
+        double w;
+        int patch, G, K, g;
+        const std::vector<int>* tiles;
+    };
+    std::vector<Run> runs;
+    size_t n = 0;            // items
+    double total = 0.0;      // their work
+
+    void add(int patch, const TileWork& tw, int G, int K, bool sat) {
+        for (size_t c = 0; c < tw.cls.size(); ++c)
+            for (int g = 0; g < G; ++g) {
+                const double w = part_work(item_work(tw, c, g, G, sat), K);
+                runs.push_back(Run{w, patch, G, K, g, &tw.cls[c]});
+                n += tw.cls[c].size() * K;
+                total += w * (double)(tw.cls[c].size() * K);
+            }
+    }
+    void sort() {
+        std::stable_sort(runs.begin(), runs.end(), [](const Run& a, const Run& b) { return a.w > b.w; });
+    }
+    // (sorted) makespan of in-order dispatch on `slots`
+    double makespan(int slots) const {
+        if (runs.empty()) return 0.0;
+        const size_t ns = (size_t)std::max(slots, 1);
+        if (n <= ns) return runs[0].w;
+        std::vector<double> heap(ns, 0.0);   // finishing times, the earliest first
+        double m = 0.0;
+        for (const Run& r : runs)
+            for (size_t k = r.tiles->size() * r.K; k > 0; --k) {
+                const double f = heap[0] + r.w;
+                m = std::max(m, f);
+                size_t i = 0;
+                for (;;) {   // f sinks to its place
+                    size_t j = 2 * i + 1;
+                    if (j >= ns) break;
+                    if (j + 1 < ns && heap[j + 1] < heap[j]) ++j;
+                    if (!(heap[j] < f)) break;
+                    heap[i] = heap[j];
+                    i = j;
+                }
+                heap[i] = f;
+            }
+        return m;
+    }
+    // No order takes less than the balanced load or the heaviest item (a
+    // little below, for the rounding of `total`).
+    double makespan_bound(int slots) const {
+        double mx = 0.0;
+        for (const Run& r : runs) mx = std::max(mx, r.w);
+        return (1.0 - 1e-9) * std::max(total / std::max(slots, 1), mx);
+    }
+    // (sorted) the items, runs of one work in patch, tile, group order
+    void expand(std::vector<TcItem>& items, std::vector<double>* work = nullptr) const {
+        items.clear();
+        items.reserve(n);
+        if (work) {
+            work->clear();
+            work->reserve(n);
+        }
+        struct Key {
+            int patch, tile, g, G, K;
+        };
+        std::vector<Key> tie;
+        for (size_t i = 0; i < runs.size();) {
+            size_t e = i;
+            tie.clear();
+            for (; e < runs.size() && runs[e].w == runs[i].w; ++e)
+                for (int t : *runs[e].tiles) tie.push_back(Key{runs[e].patch, t, runs[e].g, runs[e].G, runs[e].K});
+            if (e - i > 1)
+                std::sort(tie.begin(), tie.end(), [](const Key& a, const Key& b) {
+                    return a.patch != b.patch ? a.patch < b.patch : a.tile != b.tile ? a.tile < b.tile : a.g < b.g;
+                });
+            for (const Key& k : tie)
+                for (int q = 0; q < k.K; ++q) {
+                    items.push_back(k.K > 1 ? TcItem{k.patch, k.tile, k.g | (q << 16), k.G | (k.K << 16)}
+                                            : TcItem{k.patch, k.tile, k.g, k.G});
+                    if (work) work->push_back(runs[i].w);
+                }
+            i = e;
+        }
+    }
+};
+
 // Plan of one patch launched alone: G minimises the simulated makespan over
 // the device's resident CTA slots plus the traffic of the group-sum blend.
 // For the summed-area synthesis, gmul scales the chosen G (the autotuner's
 // search axis), within [1, gcap].
 void plan_patch(PatchHost& P, int slots, bool sat = false, double gmul = 1.0, int gcap = 16) {
-    int tiles = 0;
-    const std::vector<double> est = sat ? tile_bucket_sat(P, tiles) : tile_bucket_stages(P, tiles);
+    const TileWork tw = sat ? tile_bucket_sat(P) : tile_bucket_stages(P);
     const int nb = P.T.nb;
-    double best_cost = 0.0;
     int& groups = sat ? P.sat_groups : P.dev.groups_tc;
-    std::vector<TcItem>& plan = sat ? P.sat_items : P.tc_items;
-    auto build = [&](int G) {   // the heaviest-first plan with G groups, and its modelled cost
-        std::vector<double> work((size_t)tiles * G);
-        for (int t = 0; t < tiles; ++t)
-            for (int g = 0; g < G; ++g) work[(size_t)t * G + g] = item_work(est, nb, t, g, G, sat);
-        std::vector<int> order(work.size());
-        for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
+    const int gmax = std::max(1, std::min(std::min(nb, 16), gcap));
+    double best_cost = 0.0;
+    for (int G = 1; G <= gmax; ++G) {
+        ItemRuns r;
+        r.add(P.index, tw, G, 1, sat);
         const double blend = G <= 1 ? 0.0
                              : sat  ? kBlendUs + (G + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs
                                     : (G + 1) * 12.0 * P.T.W * P.T.H / kHbmBytesPerUs;
-        std::vector<TcItem> items;
-        for (int k : order) items.push_back(TcItem{P.index, k / G, k % G, G});
-        return std::make_pair(makespan(work, order, slots) * kStageUs + blend, items);
-    };
-    const int gmax = std::max(1, std::min(std::min(nb, 16), gcap));
-    for (int G = 1; G <= gmax; ++G) {
-        auto r = build(G);
-        if (G == 1 || r.first < best_cost) {
-            best_cost = r.first;
+        if (G > 1 && r.makespan_bound(slots) * kStageUs + blend >= best_cost) continue;
+        r.sort();
+        const double cost = r.makespan(slots) * kStageUs + blend;
+        if (G == 1 || cost < best_cost) {
+            best_cost = cost;
             groups = G;
-            plan.swap(r.second);
         }
     }
-    if (sat && gmul != 1.0) {
-        const int G = std::max(1, std::min(gmax, (int)std::lround(groups * gmul)));
-        if (G != groups) {
-            groups = G;
-            plan = build(G).second;
-        }
-    }
+    if (sat && gmul != 1.0) groups = std::max(1, std::min(gmax, (int)std::lround(groups * gmul)));
     int K = 1;
     if (sat) {
         // dense patches: split each bucket's passes over K parts when the
         // heaviest item alone would outlast the balanced share of a slot
         // (the makespan's lower bound), with at most one wave of items
-        double total = 0.0, wmax = 0.0;
-        for (const TcItem& it : plan) {
-            const double w = item_work(est, nb, it.tile, it.group, groups, true);
-            total += w;
-            wmax = std::max(wmax, w);
-        }
-        const int kwave = std::max(1, slots / std::max<int>(1, (int)plan.size()));
-        K = sat_parts_for(wmax, total / std::max(slots, 1), std::max(1, std::min(std::min(8, kwave), gcap / groups)));
-        if (K > 1) {
-            std::vector<std::pair<double, TcItem>> parts;
-            for (const TcItem& it : plan)
-                for (int q = 0; q < K; ++q)
-                    parts.push_back({part_work(item_work(est, nb, it.tile, it.group, groups, true), K),
-                                     TcItem{it.patch, it.tile, it.group | (q << 16), groups | (K << 16)}});
-            std::stable_sort(parts.begin(), parts.end(),
-                             [](const std::pair<double, TcItem>& a, const std::pair<double, TcItem>& b) {
-                                 return a.first > b.first;
-                             });
-            plan.clear();
-            for (auto& pr : parts) plan.push_back(pr.second);
-        }
+        ItemRuns whole;
+        whole.add(P.index, tw, groups, 1, true);
+        const int kwave = std::max(1, slots / std::max<int>(1, (int)whole.n));
+        K = sat_parts_for(heaviest_item(tw, groups, true), whole.total / std::max(slots, 1),
+                          std::max(1, std::min(std::min(8, kwave), gcap / groups)));
         P.sat_parts = K;
     }
+    ItemRuns r;
+    r.add(P.index, tw, groups, K, sat);
+    r.sort();
+    r.expand(sat ? P.sat_items : P.tc_items);
     (sat ? P.sat_spans : P.tc_spans) = blend_spans(P, groups * K);
 }
 
@@ -558,83 +665,95 @@ bool sat3_fits(const PatchHost& P) {
 // items runs them rather than three of single buckets (a quarter for every
 // scene: a server round of 12 scenes 1,056 us, 840 so).
 void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vector<BlendSpan>& spans,
-                  double& model_makespan, std::vector<double>& item_work_out, bool sat = false) {
+                  std::vector<double>& item_work_out, bool sat = false) {
     const size_t np = ctx->patches.size();
-    std::vector<std::vector<double>> est(np);
-    std::vector<int> tiles(np);
+    std::vector<TileWork> tw(np);
     double total = 0.0;
     for (size_t k = 0; k < np; ++k) {
-        est[k] = sat ? tile_bucket_sat(*ctx->patches[k], tiles[k]) : tile_bucket_stages(*ctx->patches[k], tiles[k]);
-        for (double e : est[k]) total += e;
-        total += (sat ? kSatItemStages : kItemStages) * tiles[k];
+        tw[k] = sat ? tile_bucket_sat(*ctx->patches[k]) : tile_bucket_stages(*ctx->patches[k]);
+        for (size_t c = 0; c < tw[k].cls.size(); ++c)
+            total += (double)tw[k].cls[c].size() * item_work(tw[k], c, 0, 1, sat);
     }
     const double per_slot = total / std::max(slots, 1);
-    auto group_work = [&](size_t k, int t, int g, int G) { return item_work(est[k], ctx->patches[k]->T.nb, t, g, G, sat); };
+    // a patch's heaviest item by G, worked out once for all shares
+    std::vector<std::vector<double>> heavy(np);
     auto heaviest = [&](size_t k, int G) {
-        double mx = 0.0;
-        for (int t = 0; t < tiles[k]; ++t)
-            for (int g = 0; g < G; ++g) mx = std::max(mx, group_work(k, t, g, G));
-        return mx;
+        while ((int)heavy[k].size() < G) heavy[k].push_back(heaviest_item(tw[k], (int)heavy[k].size() + 1, sat));
+        return heavy[k][G - 1];
     };
-    struct Plan {
-        std::vector<TcItem> items;
-        std::vector<BlendSpan> spans;
-        std::vector<double> work;
-        std::vector<int> order;
-        double makespan = 0.0, cost = 0.0;
-    } best;
-    const std::vector<double> shares = sat ? std::vector<double>{4.0, 2.0, 1.4, 1.0, 0.7, 0.5, 0.35, 0.25}
-                                           : std::vector<double>{0.25};
-    auto build = [&](double share, double gmul) {
-        const double cap = share * per_slot;
-        Plan pl;
-        double blend_us = 0.0;
+    struct Choice {
+        std::vector<int> G, K;
+    };
+    auto choose = [&](double share, double gmul) {
+        Choice ch;
         for (size_t k = 0; k < np; ++k) {
             const PatchHost& P = *ctx->patches[k];
-            const int nb = P.T.nb, gmax = std::min(std::min(nb, 16), P.partial_planes);
+            const int gmax = std::min(std::min(P.T.nb, 16), P.partial_planes);
             int G = 1;
-            while (G < gmax && heaviest(k, G) > cap) ++G;
+            while (G < gmax && heaviest(k, G) > share * per_slot) ++G;
             G = std::max(1, std::min(gmax, (int)std::lround(G * gmul)));
             // summed-area items: each bucket's passes split over K parts where
             // an item would still outlast the balanced per-slot share of the
             // frame (dense patches whose buckets take many passes)
             int K = 1;
             if (sat) K = sat_parts_for(heaviest(k, G), per_slot, std::max(1, std::min(8, P.partial_planes / G)));
-            for (int t = 0; t < tiles[k]; ++t)
-                for (int g = 0; g < G; ++g)
-                    for (int q = 0; q < K; ++q) {
-                        pl.items.push_back(K > 1 ? TcItem{P.index, t, g | (q << 16), G | (K << 16)}
-                                                 : TcItem{P.index, t, g, G});
-                        pl.work.push_back(part_work(group_work(k, t, g, G), K));
-                    }
-            const std::vector<BlendSpan> sp = blend_spans(P, G * K);
-            if (!sp.empty()) blend_us += (G * K + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs;
-            pl.spans.insert(pl.spans.end(), sp.begin(), sp.end());
+            ch.G.push_back(G);
+            ch.K.push_back(K);
         }
-        pl.order.resize(pl.items.size());
-        for (size_t k = 0; k < pl.order.size(); ++k) pl.order[k] = (int)k;
-        std::stable_sort(pl.order.begin(), pl.order.end(), [&](int a, int b) { return pl.work[a] > pl.work[b]; });
-        pl.makespan = makespan(pl.work, pl.order, slots);
-        pl.cost = pl.makespan * kStageUs + blend_us + (pl.spans.empty() ? 0.0 : kBlendUs);
-        return pl;
+        return ch;
     };
-    double share = shares[0];
-    for (double c : shares) {
-        Plan pl = build(c, 1.0);
-        if (c == shares[0] || pl.cost < best.cost) {
-            std::swap(best, pl);
-            share = c;
+    auto runs_of = [&](const Choice& ch) {
+        ItemRuns r;
+        for (size_t k = 0; k < np; ++k) r.add(ctx->patches[k]->index, tw[k], ch.G[k], ch.K[k], sat);
+        return r;
+    };
+    auto blend_cost = [&](const Choice& ch) {
+        double us = 0.0;
+        bool any = false;
+        for (size_t k = 0; k < np; ++k) {
+            const PatchHost& P = *ctx->patches[k];
+            const int planes = ch.G[k] * ch.K[k];
+            if (planes <= 1) continue;
+            us += (planes + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs;
+            any = true;
+        }
+        return us + (any ? kBlendUs : 0.0);
+    };
+    const std::vector<double> shares = sat ? std::vector<double>{4.0, 2.0, 1.4, 1.0, 0.7, 0.5, 0.35, 0.25}
+                                           : std::vector<double>{0.25};
+    double share = shares[0], best_cost = 0.0;
+    Choice best = choose(share, 1.0), last = best;
+    ItemRuns best_runs = runs_of(best);
+    best_runs.sort();
+    if (shares.size() > 1) best_cost = best_runs.makespan(slots) * kStageUs + blend_cost(best);
+    for (size_t i = 1; i < shares.size(); ++i) {
+        Choice ch = choose(shares[i], 1.0);
+        // (a share that changes nothing, or that cannot win, is not simulated)
+        if (ch.G == last.G && ch.K == last.K) continue;
+        last = ch;
+        ItemRuns r = runs_of(ch);
+        const double blend = blend_cost(ch);
+        if (r.makespan_bound(slots) * kStageUs + blend >= best_cost) continue;
+        r.sort();
+        const double cost = r.makespan(slots) * kStageUs + blend;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = std::move(ch);
+            best_runs = std::move(r);
+            share = shares[i];
         }
     }
-    if (sat && ctx->sat_gmul != 1.0) best = build(share, ctx->sat_gmul);   // the autotuner's axis
-    model_makespan = best.makespan;
-    items.clear();
-    item_work_out.clear();
-    for (int k : best.order) {
-        items.push_back(best.items[k]);
-        item_work_out.push_back(best.work[k]);
+    if (sat && ctx->sat_gmul != 1.0) {   // the autotuner's axis
+        best = choose(share, ctx->sat_gmul);
+        best_runs = runs_of(best);
+        best_runs.sort();
     }
-    spans.swap(best.spans);
+    best_runs.expand(items, &item_work_out);
+    spans.clear();
+    for (size_t k = 0; k < np; ++k) {
+        const std::vector<BlendSpan> sp = blend_spans(*ctx->patches[k], best.G[k] * best.K[k]);
+        spans.insert(spans.end(), sp.begin(), sp.end());
+    }
 }
 
 scwp_status ready(scwp_ctx* ctx) {
@@ -720,8 +839,8 @@ scwp_status sync_synth(scwp_ctx* ctx) {
     if (!ctx->d_pdevs || !ctx->d_sps) return fail(ctx, SCWP_E_NOMEM, "synthesis descriptors");
     CU(cudaMemcpyAsync(ctx->d_pdevs, pd.data(), n * sizeof(PatchDev), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(ctx->d_sps, sp.data(), n * sizeof(SynthParams), cudaMemcpyHostToDevice, ctx->st));
-    if (one_synthesis(ctx)) {
-        plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_makespan, ctx->b_work);
+    if (ctx->batched) {   // (the only mode in which the tensor-core gather runs the frame's plan)
+        plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_work);
         ctx->d_bitems = (TcItem*)dalloc(ctx, std::max<size_t>(1, ctx->b_items.size()) * sizeof(TcItem));
         ctx->d_bspans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, ctx->b_spans.size()) * sizeof(BlendSpan));
         if (!ctx->d_bitems || !ctx->d_bspans) return fail(ctx, SCWP_E_NOMEM, "batched plan");
@@ -730,7 +849,9 @@ scwp_status sync_synth(scwp_ctx* ctx) {
         if (!ctx->b_spans.empty())
             CU(cudaMemcpyAsync(ctx->d_bspans, ctx->b_spans.data(), ctx->b_spans.size() * sizeof(BlendSpan),
                                cudaMemcpyHostToDevice, ctx->st));
-        plan_batched(ctx, ctx->sat_slots, ctx->s_items, ctx->s_spans, ctx->s_makespan, ctx->s_work, true);
+    }
+    if (one_synthesis(ctx)) {
+        plan_batched(ctx, ctx->sat_slots, ctx->s_items, ctx->s_spans, ctx->s_work, true);
         ctx->d_sitems = (TcItem*)dalloc(ctx, std::max<size_t>(1, ctx->s_items.size()) * sizeof(TcItem));
         ctx->d_sspans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, ctx->s_spans.size()) * sizeof(BlendSpan));
         if (!ctx->d_sitems || !ctx->d_sspans) return fail(ctx, SCWP_E_NOMEM, "batched plan");
@@ -997,8 +1118,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
         // can split into parts
         int gpart = std::min(nbmax, 2 * gsat);
         double max_passes = 0.0;
-        int tiles_est = 0;
-        tile_bucket_sat(*P, tiles_est, &max_passes);
+        const int tiles_sat = tile_bucket_sat(*P, &max_passes).tiles;
         if (max_passes >= 2.0 && (size_t)64 * 12 * T.W * T.H <= ((size_t)256 << 20)) gpart = 64;
         P->partial_planes = std::max(std::max(D.groups, D.groups_tc), gpart);
         const int variant = (ctx->sat_variant == 1 && P->sat3_ok) ? 1 : 0;
@@ -1007,8 +1127,6 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
         plan_patch(*P, P->sat_slots, true, ctx->sat_gmul, P->partial_planes);
         P->d_items = (TcItem*)dalloc(ctx, P->tc_items.size() * sizeof(TcItem));
         P->d_spans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, P->tc_spans.size()) * sizeof(BlendSpan));
-        int tiles_sat = 0;
-        tile_bucket_sat(*P, tiles_sat);
         P->sat_item_cap = tiles_sat * P->partial_planes;   // G K <= the planes
         P->d_sat_items = (TcItem*)dalloc(ctx, (size_t)P->sat_item_cap * sizeof(TcItem));
         P->d_sat_spans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, blend_spans(*P, 2).size()) * sizeof(BlendSpan));

@@ -1,0 +1,90 @@
+"""When and how often a frame's plan is made: for the mode that runs, once the
+scene has changed, in device memory that is reused."""
+import numpy as np
+import pytest
+
+from oracle.scene import OracleScene
+from paper_2511_02852_gb300 import workloads as wl
+from test_gpu_parity import compare_maps
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    yield
+    torch.cuda.synchronize()
+
+
+def _cfg(n=4, nb=12):
+    rng = np.random.default_rng(n)
+    spec = wl.spectrum(wind_speed=9.0, fetch=40e3, n_buckets=nb, n_theta=8, fft_n=64, fft_L=120.0, seed=11)
+    ps = [wl.patch(origin_x=5.0 * i, cell=0.5, width=int(rng.integers(60, 300)), height=int(rng.integers(60, 300)),
+                   max_particles=8000, prefill=2000) for i in range(n)]
+    return wl.scene("plan", spec, ps, frames=2)
+
+
+class _Counted:
+    """A scene whose allocator calls are counted."""
+
+    def __init__(self, cfg):
+        from paper_2511_02852_gb300 import scwp
+        self.calls = self.held = 0
+        self.sizes = {}
+        orig_alloc = torch.cuda.caching_allocator_alloc
+        orig_free = torch.cuda.caching_allocator_delete
+
+        def alloc(nbytes, device, stream):
+            p = orig_alloc(nbytes, device, stream)
+            self.calls += 1
+            self.held += nbytes
+            self.sizes[int(p)] = nbytes
+            return p
+
+        def free(p):
+            self.held -= self.sizes.pop(int(p), 0)
+            orig_free(p)
+
+        torch.cuda.caching_allocator_alloc, torch.cuda.caching_allocator_delete = alloc, free
+        self._undo = (orig_alloc, orig_free)
+        self.sc = scwp.Scene(cfg, device=0)
+
+    def close(self):
+        self.sc.close()
+        torch.cuda.caching_allocator_alloc, torch.cuda.caching_allocator_delete = self._undo
+
+
+def test_a_plain_scene_makes_no_tensor_core_plan():
+    """Descriptors, parameters and the summed-area frame plan: four blocks at
+    most; the tensor-core frame plan is made once the scene is batched."""
+    cfg = _cfg()
+    c = _Counted(cfg)
+    try:
+        before = c.calls
+        c.sc.step(cfg["dt"])
+        torch.cuda.synchronize()
+        assert c.calls - before <= 4
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("first_batched", [False, True])
+def test_modes_in_turn(first_batched):
+    """Either synthesis, in either mode, whichever came first."""
+    from paper_2511_02852_gb300 import scwp
+    cfg = _cfg()
+    sc, orc = scwp.Scene(cfg, device=0), OracleScene(cfg)
+    sc.step(cfg["dt"])
+    orc.step(cfg["dt"])
+    bg = orc.background()
+    ref = [orc.patch_maps(p, bg)[0] for p in range(len(cfg["patches"]))]
+    for batched in (first_batched, not first_batched):
+        sc.set_batched(batched)
+        for mode in (scwp.SYNTH_GATHER, scwp.SYNTH_SAT, scwp.SYNTH_GATHER):
+            sc.resynthesize(mode)
+            for p, r in enumerate(ref):
+                compare_maps(sc.maps(p), r, orc.spec.Hs(), "batched %d mode %d patch %d" % (batched, mode, p))
+    sc.close()
