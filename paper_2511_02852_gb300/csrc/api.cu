@@ -130,6 +130,8 @@ struct scwp_ctx {
     bool synth_dirty = true;
     int b_lo = 0, b_hi = 1 << 30;     // buckets synthesised by the tensor-core modes
     int slots = 0;
+    unsigned char* d_synth = nullptr; // the block that holds them and the frame's plans (sync_synth)
+    size_t synth_cap = 0;
     PatchDev* d_pdevs = nullptr;
     SynthParams* d_sps = nullptr;
     std::vector<TcItem> b_items;
@@ -191,6 +193,15 @@ void* dalloc(scwp_ctx* c, size_t bytes) {
         c->alloc_bytes += bytes;
     }
     return p;
+}
+
+// give back one block of `bytes` bytes (nothing may still use it)
+void dfree(scwp_ctx* c, void* p, size_t bytes) {
+    if (!p) return;
+    c->allocs.erase(std::remove(c->allocs.begin(), c->allocs.end(), p), c->allocs.end());
+    c->alloc_bytes -= (bytes + 255) & ~(size_t)255;
+    if (c->d.free) c->d.free(p, c->d.alloc_user);
+    else cudaFree(p);
 }
 
 void dfree_all(scwp_ctx* c) {
@@ -821,8 +832,11 @@ const PatchDev* patch_devs(scwp_ctx* ctx) {
 // side took 243 us a frame so, 160 with the frame's plan.
 bool one_synthesis(const scwp_ctx* ctx) { return ctx->batched || ctx->patches.size() > 1; }
 
+size_t align16(size_t n) { return (n + 15) & ~(size_t)15; }
+
 // device copies of the patch descriptors and synthesis parameters (and the
-// batched plan) after the set of patches or the batching mode changed
+// frame's plans) after the set of patches, the batching mode or the plans'
+// parameters changed: one block, kept while they fit in it, and one copy
 scwp_status sync_synth(scwp_ctx* ctx) {
     if (!ctx->synth_dirty) return SCWP_OK;
     const size_t n = ctx->patches.size();
@@ -834,34 +848,41 @@ scwp_status sync_synth(scwp_ctx* ctx) {
         pd[k] = ctx->patches[k]->dev;
         sp[k] = synth_params(ctx, *ctx->patches[k]);
     }
-    ctx->d_pdevs = (PatchDev*)dalloc(ctx, std::max<size_t>(1, n) * sizeof(PatchDev));
-    ctx->d_sps = (SynthParams*)dalloc(ctx, std::max<size_t>(1, n) * sizeof(SynthParams));
-    if (!ctx->d_pdevs || !ctx->d_sps) return fail(ctx, SCWP_E_NOMEM, "synthesis descriptors");
-    CU(cudaMemcpyAsync(ctx->d_pdevs, pd.data(), n * sizeof(PatchDev), cudaMemcpyHostToDevice, ctx->st));
-    CU(cudaMemcpyAsync(ctx->d_sps, sp.data(), n * sizeof(SynthParams), cudaMemcpyHostToDevice, ctx->st));
-    if (ctx->batched) {   // (the only mode in which the tensor-core gather runs the frame's plan)
-        plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_work);
-        ctx->d_bitems = (TcItem*)dalloc(ctx, std::max<size_t>(1, ctx->b_items.size()) * sizeof(TcItem));
-        ctx->d_bspans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, ctx->b_spans.size()) * sizeof(BlendSpan));
-        if (!ctx->d_bitems || !ctx->d_bspans) return fail(ctx, SCWP_E_NOMEM, "batched plan");
-        CU(cudaMemcpyAsync(ctx->d_bitems, ctx->b_items.data(), ctx->b_items.size() * sizeof(TcItem),
-                           cudaMemcpyHostToDevice, ctx->st));
-        if (!ctx->b_spans.empty())
-            CU(cudaMemcpyAsync(ctx->d_bspans, ctx->b_spans.data(), ctx->b_spans.size() * sizeof(BlendSpan),
-                               cudaMemcpyHostToDevice, ctx->st));
+    // (batched mode is the only one in which the tensor-core gather runs the frame's plan)
+    ctx->b_items.clear();
+    ctx->b_spans.clear();
+    ctx->s_items.clear();
+    ctx->s_spans.clear();
+    if (ctx->batched) plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_work);
+    if (one_synthesis(ctx)) plan_batched(ctx, ctx->sat_slots, ctx->s_items, ctx->s_spans, ctx->s_work, true);
+    std::vector<unsigned char> h;
+    auto put = [&](const auto& v) {   // v's place in the block
+        const size_t o = h.size(), bytes = v.size() * sizeof(v[0]);
+        h.resize(o + align16(std::max<size_t>(1, bytes)));
+        if (bytes) memcpy(h.data() + o, v.data(), bytes);
+        return o;
+    };
+    const size_t o_pd = put(pd), o_sp = put(sp);
+    const size_t o_bi = put(ctx->b_items), o_bs = put(ctx->b_spans);
+    const size_t o_si = put(ctx->s_items), o_ss = put(ctx->s_spans);
+    if (ctx->synth_cap < h.size()) {
+        // frames in flight may still read the old block; the new one has
+        // room for the larger plans of other settings
+        if (ctx->d_synth) CU(cudaStreamSynchronize(ctx->st));
+        dfree(ctx, ctx->d_synth, ctx->synth_cap);
+        ctx->synth_cap = 0;
+        ctx->d_synth = (unsigned char*)dalloc(ctx, 2 * h.size());
+        if (!ctx->d_synth) return fail(ctx, SCWP_E_NOMEM, "synthesis descriptors and plans");
+        ctx->synth_cap = 2 * h.size();
     }
-    if (one_synthesis(ctx)) {
-        plan_batched(ctx, ctx->sat_slots, ctx->s_items, ctx->s_spans, ctx->s_work, true);
-        ctx->d_sitems = (TcItem*)dalloc(ctx, std::max<size_t>(1, ctx->s_items.size()) * sizeof(TcItem));
-        ctx->d_sspans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, ctx->s_spans.size()) * sizeof(BlendSpan));
-        if (!ctx->d_sitems || !ctx->d_sspans) return fail(ctx, SCWP_E_NOMEM, "batched plan");
-        CU(cudaMemcpyAsync(ctx->d_sitems, ctx->s_items.data(), ctx->s_items.size() * sizeof(TcItem),
-                           cudaMemcpyHostToDevice, ctx->st));
-        if (!ctx->s_spans.empty())
-            CU(cudaMemcpyAsync(ctx->d_sspans, ctx->s_spans.data(), ctx->s_spans.size() * sizeof(BlendSpan),
-                               cudaMemcpyHostToDevice, ctx->st));
-    }
-    // the host vectors are copied before they go out of scope
+    ctx->d_pdevs = reinterpret_cast<PatchDev*>(ctx->d_synth + o_pd);
+    ctx->d_sps = reinterpret_cast<SynthParams*>(ctx->d_synth + o_sp);
+    ctx->d_bitems = reinterpret_cast<TcItem*>(ctx->d_synth + o_bi);
+    ctx->d_bspans = reinterpret_cast<BlendSpan*>(ctx->d_synth + o_bs);
+    ctx->d_sitems = reinterpret_cast<TcItem*>(ctx->d_synth + o_si);
+    ctx->d_sspans = reinterpret_cast<BlendSpan*>(ctx->d_synth + o_ss);
+    CU(cudaMemcpyAsync(ctx->d_synth, h.data(), h.size(), cudaMemcpyHostToDevice, ctx->st));
+    // the host copy is read before it goes out of scope
     CU(cudaStreamSynchronize(ctx->st));
     ctx->synth_dirty = false;
     return SCWP_OK;
@@ -1470,7 +1491,9 @@ static scwp_status run_graph(scwp_ctx* ctx, FrameGraph& G, const std::vector<Inj
     if (g < 0) g = !G.valid[0] ? 0 : 1;
     const size_t bytes = 16 + ips.size() * sizeof(InjectParams);
     if (!G.dparams || G.bytes < bytes) {
-        graph_reset(G);
+        graph_reset(G);   // (its replays are done)
+        dfree(ctx, G.dparams, G.bytes);
+        G.bytes = 0;
         G.dparams = (unsigned char*)dalloc(ctx, bytes);
         if (!G.dparams) return fail(ctx, SCWP_E_NOMEM, "graph parameters");
         for (int k = 0; k < 2; ++k) {
@@ -2278,8 +2301,6 @@ void sv_free(scwp_server* sv, void* p) {
     if (sv->d.free) sv->d.free(p, sv->d.alloc_user);
     else cudaFree(p);
 }
-
-size_t align16(size_t n) { return (n + 15) & ~(size_t)15; }
 
 }  // namespace
 

@@ -88,3 +88,47 @@ def test_modes_in_turn(first_batched):
             for p, r in enumerate(ref):
                 compare_maps(sc.maps(p), r, orc.spec.Hs(), "batched %d mode %d patch %d" % (batched, mode, p))
     sc.close()
+
+
+def test_the_first_frame_takes_one_block():
+    cfg = _cfg()
+    c = _Counted(cfg)
+    try:
+        before = c.calls
+        c.sc.step(cfg["dt"])
+        torch.cuda.synchronize()
+        assert c.calls - before <= 1
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_planning_again_holds_no_more_memory(batched):
+    """A second round of the same settings takes no device memory that the
+    first did not."""
+    cfg = _cfg()
+    c = _Counted(cfg)
+    try:
+        sc = c.sc
+        sc.set_batched(batched)
+
+        def settings():
+            for lo, hi in ((0, 3), (3, 12), (0, 64)):
+                sc.set_bucket_range(lo, hi)
+                sc.step(cfg["dt"])
+            for gmul in (0.5, 2.0, 8.0, 1.0):
+                sc.set_sat_plan(0, gmul)
+                sc.step(cfg["dt"])
+            sc.set_batched(not batched)
+            sc.step(cfg["dt"])
+            sc.set_batched(batched)
+            sc.step(cfg["dt"])
+            torch.cuda.synchronize()
+
+        settings()
+        held = c.held
+        for _ in range(3):
+            settings()
+            assert c.held == held
+    finally:
+        c.close()
