@@ -179,8 +179,10 @@ typedef struct scwp_patch_info {
     int32_t synth_groups;      /* bucket groups of the tensor-core synthesis (planned at creation) */
     int32_t synth_items;       /* its (tile, group) work items = CTAs per synthesis launch */
     int32_t synth_slots;       /* resident CTA slots of the device the plan assumed */
-    int32_t sat_groups;        /* bucket groups of the summed-area synthesis */
-    int32_t sat_items;         /* its (tile, group) work items */
+    int32_t sat_groups;        /* bucket groups of the summed-area synthesis: of the frame's
+                                  plan with several patches or in batched mode, else of the
+                                  patch's own */
+    int32_t sat_items;         /* its (tile, group, part) work items in that plan */
     int32_t sat_slots;         /* resident CTA slots its plan assumed */
     int32_t frame_param_bytes; /* host-computed plan of one frame of this patch (injection
                                   counts, host-placed spawn points) copied to the device */

@@ -68,6 +68,8 @@ struct PatchHost {
     int sat_slots = 0;
     int sat_item_cap = 0;             // capacity of d_sat_items (items of the largest G)
     int sat_parts = 1;                // parts each bucket's passes are split over (dense patches)
+    int frame_groups = 1, frame_parts = 1;   // its bucket groups and parts in the frame's summed-area plan
+    int frame_items = 0;                     // its items there
     bool sat3_ok = false;             // every bucket fits the three-group kernel's row table
 };
 
@@ -127,7 +129,8 @@ struct scwp_ctx {
     // tensor-core synthesis: patch descriptors and parameters on the device,
     // and the batched plan (all patches in one launch)
     bool batched = false;
-    bool synth_dirty = true;
+    bool synth_dirty = true;          // the device copies below are out of date
+    bool plan_dirty = true;           // so are the frame's plans
     int b_lo = 0, b_hi = 1 << 30;     // buckets synthesised by the tensor-core modes
     int slots = 0;
     unsigned char* d_synth = nullptr; // the block that holds them and the frame's plans (sync_synth)
@@ -762,6 +765,12 @@ void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vec
     best_runs.expand(items, &item_work_out);
     spans.clear();
     for (size_t k = 0; k < np; ++k) {
+        if (sat) {
+            PatchHost& P = *ctx->patches[k];
+            P.frame_groups = best.G[k];
+            P.frame_parts = best.K[k];
+            P.frame_items = tw[k].tiles * best.G[k] * best.K[k];
+        }
         const std::vector<BlendSpan> sp = blend_spans(*ctx->patches[k], best.G[k] * best.K[k]);
         spans.insert(spans.end(), sp.begin(), sp.end());
     }
@@ -834,6 +843,20 @@ bool one_synthesis(const scwp_ctx* ctx) { return ctx->batched || ctx->patches.si
 
 size_t align16(size_t n) { return (n + 15) & ~(size_t)15; }
 
+// The frame's plans, on the host, after the set of patches, the batching mode
+// or the plans' parameters changed.
+void plan_frame(scwp_ctx* ctx) {
+    if (!ctx->plan_dirty) return;
+    ctx->b_items.clear();
+    ctx->b_spans.clear();
+    ctx->s_items.clear();
+    ctx->s_spans.clear();
+    // (batched mode is the only one in which the tensor-core gather runs the frame's plan)
+    if (ctx->batched) plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_work);
+    if (one_synthesis(ctx)) plan_batched(ctx, ctx->sat_slots, ctx->s_items, ctx->s_spans, ctx->s_work, true);
+    ctx->plan_dirty = false;
+}
+
 // device copies of the patch descriptors and synthesis parameters (and the
 // frame's plans) after the set of patches, the batching mode or the plans'
 // parameters changed: one block, kept while they fit in it, and one copy
@@ -848,13 +871,7 @@ scwp_status sync_synth(scwp_ctx* ctx) {
         pd[k] = ctx->patches[k]->dev;
         sp[k] = synth_params(ctx, *ctx->patches[k]);
     }
-    // (batched mode is the only one in which the tensor-core gather runs the frame's plan)
-    ctx->b_items.clear();
-    ctx->b_spans.clear();
-    ctx->s_items.clear();
-    ctx->s_spans.clear();
-    if (ctx->batched) plan_batched(ctx, ctx->slots, ctx->b_items, ctx->b_spans, ctx->b_work);
-    if (one_synthesis(ctx)) plan_batched(ctx, ctx->sat_slots, ctx->s_items, ctx->s_spans, ctx->s_work, true);
+    plan_frame(ctx);
     std::vector<unsigned char> h;
     auto put = [&](const auto& v) {   // v's place in the block
         const size_t o = h.size(), bytes = v.size() * sizeof(v[0]);
@@ -1250,7 +1267,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
     P->energy.assign(T.nb, 0.0);
     graph_reset(ctx);
     ctx->patches.push_back(P);
-    ctx->synth_dirty = true;
+    ctx->synth_dirty = ctx->plan_dirty = true;
     if (patch_id) *patch_id = P->index;
     // velocity tables for the current dt (a provisional 1/60 s before the
     // first step, so the trough offsets are valid for scwp_resynthesize)
@@ -1632,7 +1649,7 @@ scwp_status scwp_set_batched(scwp_ctx* ctx, int32_t on) {
     if (s != SCWP_OK) return s;
     graph_reset(ctx);
     ctx->batched = on != 0;
-    ctx->synth_dirty = true;
+    ctx->synth_dirty = ctx->plan_dirty = true;
     return SCWP_OK;
 }
 
@@ -1676,7 +1693,7 @@ static scwp_status replan_sat(scwp_ctx* ctx) {
     }
     CU(cudaStreamSynchronize(ctx->st));
     graph_reset(ctx);
-    ctx->synth_dirty = true;
+    ctx->synth_dirty = ctx->plan_dirty = true;
     return SCWP_OK;
 }
 
@@ -1956,6 +1973,7 @@ scwp_status scwp_patch_info_get(scwp_ctx* ctx, int32_t patch_id, scwp_patch_info
     if (s != SCWP_OK) return s;
     if (!out || patch_id < 0 || patch_id >= (int)ctx->patches.size()) return fail(ctx, SCWP_E_INVALID, "args");
     const PatchHost* P = ctx->patches[patch_id];
+    if (one_synthesis(ctx)) plan_frame(ctx);
     memset(out, 0, sizeof(*out));
     out->n_buckets = P->T.nb;
     out->n_theta = P->T.nth;
@@ -1968,11 +1986,13 @@ scwp_status scwp_patch_info_get(scwp_ctx* ctx, int32_t patch_id, scwp_patch_info
     out->synth_groups = P->dev.groups_tc;
     out->synth_items = (int32_t)P->tc_items.size();
     out->synth_slots = P->tc_slots;
-    out->sat_groups = P->sat_groups;
-    out->sat_items = (int32_t)P->sat_items.size();
+    // the summed-area plan that runs: the frame's, or the patch's own
+    const bool frame = one_synthesis(ctx);
+    out->sat_groups = frame ? P->frame_groups : P->sat_groups;
+    out->sat_items = frame ? P->frame_items : (int32_t)P->sat_items.size();
     out->sat_slots = P->sat_slots;
     out->sat_variant = (ctx->sat_variant == 1 && P->sat3_ok) ? 1 : 0;
-    out->sat_parts = P->sat_parts;
+    out->sat_parts = frame ? P->frame_parts : P->sat_parts;
     out->frame_param_bytes = (int32_t)sizeof(InjectParams);
     for (int i = 0; i < P->T.nb; ++i) {
         out->bin_cells[i] = P->bin_cells[i];

@@ -132,3 +132,36 @@ def test_planning_again_holds_no_more_memory(batched):
             assert c.held == held
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("n,side", [(1, 300), (2, 100), (32, 512)])
+def test_patch_info_describes_the_plan_that_runs(n, side, batched):
+    """A group-sum blend runs if and only if some patch has more than one
+    plane, and every patch has one item per tile, group and part."""
+    from paper_2511_02852_gb300 import scwp
+    spec = wl.spectrum(wind_speed=9.0, fetch=40e3, n_buckets=12, n_theta=8, fft_n=64, fft_L=120.0, seed=11)
+    cfg = wl.scene("info", spec, [wl.patch(cell=0.5, width=side, height=side, max_particles=4000, prefill=500)
+                                  for _ in range(n)], frames=1)
+    sc = scwp.Scene(cfg, device=0)
+    sc.set_batched(batched)
+    count = lambda: scwp_launches(scwp, sc)
+    sc.step(cfg["dt"])
+    for gmul in (1.0, 8.0, 0.125):
+        sc.set_sat_plan(0, gmul)
+        infos = [sc.info(p) for p in range(n)]
+        before = count()
+        sc.resynthesize(scwp.SYNTH_SAT)
+        passes = (int(infos[0].total_bins).bit_length() + 7) // 8
+        blend = any(i.sat_groups * i.sat_parts > 1 for i in infos)
+        assert count() - before == 1 + passes + 1 + 1 + blend   # keys, sort, records, synthesis, blend
+        for i in infos:
+            assert i.sat_items == ((side + 63) // 64) ** 2 * i.sat_groups * i.sat_parts
+    sc.close()
+
+
+def scwp_launches(scwp, sc):
+    import ctypes
+    n = ctypes.c_int64()
+    assert scwp.lib().scwp_launch_count(sc.ctx, ctypes.byref(n)) == 0
+    return n.value
