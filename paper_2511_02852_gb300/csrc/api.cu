@@ -675,9 +675,9 @@ bool sat3_fits(const PatchHost& P) {
 // quarter for the tensor-core gather), and all items of all patches run
 // heaviest first.  For the summed-area synthesis the share is the one, of a
 // few, with the smallest modelled makespan and blend: an item's start and
-// store cost more than half a pass, so a scene that fits one wave of longer
-// items runs them rather than three of single buckets (a quarter for every
-// scene: a server round of 12 scenes 1,056 us, 840 so).
+// store cost nearly half a pass (2.6 of 5.7 us), so a scene that fits one wave
+// of longer items runs them rather than three of single buckets (a quarter for
+// every scene: a server round of 12 scenes 1,056 us, 840 so).
 void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vector<BlendSpan>& spans,
                   std::vector<double>& item_work_out, bool sat = false) {
     const size_t np = ctx->patches.size();
@@ -1099,7 +1099,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
         D.vals[k] = (uint32_t*)dalloc(ctx, 2 * cap * 4);
         ok = ok && D.x[k] && D.y[k] && D.bd[k] && D.keys[k] && D.vals[k];
     }
-    D.count = (int32_t*)dalloc(ctx, 2 * sizeof(int32_t));
+    D.count = (int32_t*)dalloc(ctx, 4 * sizeof(int32_t));
     D.blk = (uint32_t*)dalloc(ctx, ((size_t)D.nblk_c + 1) * 4);
     const size_t ng = (size_t)T.nb * T.nth;
     D.vq = (int4*)dalloc(ctx, (ng + (D.emitter ? kWakeDirs : 0)) * sizeof(int4));
@@ -1215,7 +1215,7 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
     }
     int32_t n0 = (int32_t)std::min<size_t>(px.size(), cap);
     uint64_t flags0 = px.size() > cap ? kErrCapacity : 0;
-    int32_t counts[2] = {n0, n0};
+    int32_t counts[4] = {n0, n0, 0, 0};
     CU(cudaMemcpyAsync(D.amp, ampf.data(), ng * sizeof(float), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(D.bk, P->bk.data(), T.nb * sizeof(BucketDev), cudaMemcpyHostToDevice, ctx->st));
     CU(cudaMemcpyAsync(P->d_items, P->tc_items.data(), P->tc_items.size() * sizeof(TcItem), cudaMemcpyHostToDevice,

@@ -52,7 +52,8 @@ struct PatchDev {
     int32_t* x[2] = {nullptr, nullptr};
     int32_t* y[2] = {nullptr, nullptr};
     uint32_t* bd[2] = {nullptr, nullptr}; // bucket << 16 | direction
-    int32_t* count = nullptr;             // [0] live, [1] live after compaction
+    int32_t* count = nullptr;             // [4]: live, live after compaction, the look-backs that have run
+                                          // out (bits; the patch is then empty), unused
     uint32_t* blk = nullptr;              // [nblk_c + 1] look-back words of the step's tiles, its ticket
                                           // (zero between frames: the record pass clears them)
     int nblk_c = 0;
@@ -174,11 +175,12 @@ void count_launches(int n);
 // pdl_enter() before touching global memory, which waits until the
 // predecessor grid has completed (its writes visible) and then allows the
 // successor grid to be scheduled.  Only the launch latency overlaps: no
-// kernel reads or writes anything before its predecessor is done.  Launches
-// recorded into a CUDA graph go without it: a replayed graph has no launch
-// latency to hide, and with several patches' streams in one graph the early
-// blocks only held SM slots (batched frames 1.6% slower with it).  Without
-// the attribute pdl_enter() returns at once.
+// kernel reads or writes anything that its predecessor may write before that
+// one is done.  Launches recorded into a CUDA graph go without it.  (That was
+// measured with a stream per patch in the graph, whose early blocks only held
+// SM slots: batched frames 1.6 % slower with it.  As one chain, which a frame
+// is now, it has not been measured.)  Without the attribute pdl_enter()
+// returns at once.
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -119,12 +119,22 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* a) {
 // past the key buffers, the records would be gathered by ids from places that
 // nothing wrote, and the synthesis would follow bin offsets that run backwards.
 // From the kernel after the one that gave up on, the patch is empty instead:
-// no keys, every bin offset zero.  A kernel with such waits reads the count in
-// one thread for its block, as the flag may be set while it runs.
-__device__ __forceinline__ int live_count(const PatchDev& p) {
-    const unsigned long long err = p.stats[2];
-    const int n = p.count[0];   // (both loads in flight together)
-    return (err & kErrTimeout) ? 0 : n;
+// no keys, every bin offset zero.
+// count[2] holds a bit for each kernel of a frame that may give up, and one
+// for an earlier frame (set by the record pass).  A kernel looks only at the
+// bits of kernels before it, so that all its threads see the same count; the
+// bits come with the count in one load.
+constexpr int kGaveUpStep = 1, kGaveUpBefore = 1 << 8, kGaveUpAny = ~0;
+__host__ __device__ constexpr int gave_up_pass(int ps) { return 2 << ps; }
+static_assert(gave_up_pass(kMaxSortPasses - 1) < kGaveUpBefore, "one bit each");
+
+__device__ __forceinline__ int live_count(const PatchDev& p, int gave_up) {
+    const int4 c = *reinterpret_cast<const int4*>(p.count);
+    return (c.z & gave_up) ? 0 : c.x;
+}
+__device__ __forceinline__ void give_up(const PatchDev& p, int bit) {
+    atomicOr(&p.stats[2], (unsigned long long)kErrTimeout);
+    atomicOr(&p.count[2], bit);
 }
 
 // ---- a6: bin keys -------------------------------------------------------------
@@ -255,23 +265,19 @@ __global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack
                                                int first_tile) {
     __shared__ KeyCounts C;
     __shared__ uint32_t s_cnt[32], s_off;   // survivors of 32-particle runs, then the runs' offsets
-    __shared__ int s_bid, s_n;
+    __shared__ int s_bid;
     static_assert(kItems * kTpb / 32 == 32, "one run per lane of the scanning warp");
     const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
     if (M > 1 && (int)blockIdx.x >= p.nblk_c) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t* const words = p.blk;          // [nblk_c] look-back words, then the ticket
-    if (tid == 0) {
-        const int t = (int)atomicAdd(words + p.nblk_c, 1u);   // (in flight beside the count)
-        s_n = live_count(p);
-        s_bid = t + first_tile;
-    }
+    if (tid == 0) s_bid = (int)atomicAdd(words + p.nblk_c, 1u) + first_tile;
     clear_sort_words(p);
     keys_begin(C, p);
     __syncthreads();
     const int bid = s_bid;
-    const int n = s_n, base = bid * kTileC;
+    const int n = live_count(p, kGaveUpBefore), base = bid * kTileC;
     if (base >= n) {   // (uniform)
         if (n == 0 && bid == 0 && tid == 0) p.count[0] = p.count[1] = 0;
         return;
@@ -339,7 +345,7 @@ __global__ void __launch_bounds__(kTpb) k_step(const __grid_constant__ PatchPack
                 if (lane == 0 && fu < 32) late = clock64() - t0 > wait_cycles;
                 if (__any_sync(0xffffffffu, late)) {
                     // (excl is then below the true offset: every store stays in bounds)
-                    if (lane == 0) atomicOr(&p.stats[2], (unsigned long long)kErrTimeout);
+                    if (lane == 0) give_up(p, kGaveUpStep);
                     break;
                 }
             }
@@ -499,7 +505,7 @@ __global__ void __launch_bounds__(kTpb) k_bin_keys(const __grid_constant__ Patch
     pdl_enter();
     if (M > 1 && (int)blockIdx.x >= p.nblk_s) return;
     clear_sort_words(p);
-    const int n = live_count(p);
+    const int n = live_count(p, kGaveUpAny);
     const int32_t* X = p.x[p.cur];
     const int32_t* Y = p.y[p.cur];
     const uint32_t* BD = p.bd[p.cur];
@@ -597,7 +603,7 @@ __global__ void __launch_bounds__(kSortTpb, 3) k_sort_pass(const __grid_constant
     __shared__ uint32_t s_ls[256];              // the digit's first position in the reordered tile
     __shared__ uint32_t s_gb[256];              // output position of reordered tile position 0 of the digit
     __shared__ uint32_t s_warp[8];
-    __shared__ int s_bid, s_n;
+    __shared__ int s_bid;
     __shared__ bool s_last;
     const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
@@ -610,12 +616,9 @@ __global__ void __launch_bounds__(kSortTpb, 3) k_sort_pass(const __grid_constant
     uint32_t* const dtot = p.hist + 256 * ps;
     uint32_t* const status = p.sort_status + (size_t)ps * p.nblk_o * 256;
     uint32_t* const ticket = p.sort_ticket + 2 * ps;
-    unsigned long long* const err = p.stats + 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t dt = tid < 256 ? dtot[tid] : 0u;
-    if (tid == 0) s_n = 2 * live_count(p);   // (read after the scan's barrier)
-    const uint32_t gd = block_exscan256(dt, s_warp);   // keys of smaller digits, all tiles
-    const int n = s_n;
+    const int n = 2 * live_count(p, kGaveUpBefore | (gave_up_pass(ps) - 1));
+    const uint32_t gd = block_exscan256(tid < 256 ? dtot[tid] : 0u, s_warp);   // keys of smaller digits, all tiles
     const uint32_t lt = (1u << lane) - 1u;
     for (;;) {
         if (tid == 0) s_bid = (int)atomicAdd(ticket, 1u) + first_tile;
@@ -687,7 +690,7 @@ __global__ void __launch_bounds__(kSortTpb, 3) k_sort_pass(const __grid_constant
                     }
                     if (done) break;
                     if (stalled && clock64() - t0 > wait_cycles) {
-                        atomicOr(err, (unsigned long long)kErrTimeout);
+                        give_up(p, gave_up_pass(ps));
                         break;
                     }
                 }
@@ -775,7 +778,6 @@ __global__ void __launch_bounds__(kTpb) k_offsets_records(const __grid_constant_
     __shared__ uint4 s_rec[kTpb / 32][64];
     const PatchDev& p = pk.p[M == 1 ? 0 : blockIdx.y];
     pdl_enter();
-    const int n = 2 * live_count(p);
     const uint32_t* const keys = p.keys[sort_passes(p) & 1];
     const uint32_t* const vals = p.vals[sort_passes(p) & 1];
     // the frame's statistics (the error flags stay; the synthesis counts its
@@ -796,6 +798,8 @@ __global__ void __launch_bounds__(kTpb) k_offsets_records(const __grid_constant_
         if (t == p.nb) p.stats[3 + p.nb] = p.stats[5 + p.nb] = 0ull;
     }
     for (int i = blockIdx.x * kTpb + threadIdx.x; i <= p.nblk_c; i += gridDim.x * kTpb) p.blk[i] = 0u;
+    const int n = 2 * live_count(p, kGaveUpAny);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && n == 0 && p.count[2]) p.count[2] = kGaveUpBefore;
     const int4* PK = p.pk;
     const uint32_t tb = (uint32_t)p.total_bins;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
