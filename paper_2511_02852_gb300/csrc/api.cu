@@ -1603,10 +1603,14 @@ static scwp_status step_impl(scwp_ctx* ctx, double dt) {
     scwp_status s = frame_begin(ctx, dt);
     if (s != SCWP_OK) return s;
     // batched frames of several patches replay a captured graph unless
-    // stage timing is on.  A one-patch frame (about 13 kernels) runs eagerly
-    // instead: chained by programmatic dependent launch it measured faster
-    // than the replay (0.308 against 0.317-0.322 ms on a 1024^2 patch with
-    // 200k particles), whose staged-parameter copy heads the frame.
+    // stage timing is on.  A one-patch frame (eight or nine kernels) runs
+    // eagerly instead: chained by programmatic dependent launch it measured
+    // faster than the replay (0.308 against 0.317-0.322 ms on a 1024^2 patch
+    // with 200k particles, when a frame had about 13 kernels), whose
+    // staged-parameter copy heads the frame.  With several patches the two
+    // are close (replay / eager: 2.163 / 2.157 ms for 32 patches of 4M
+    // particles, 6.33 / 6.37 for 8 of 2M each, 0.168 / 0.157 for four of up to
+    // 500 cells a side), and the replay leaves the host free.
     if (ctx->batched && !ctx->timing && ctx->patches.size() > 1 && ctx->patches.size() <= 64 &&
         (ctx->synth_mode == SCWP_SYNTH_GATHER || ctx->synth_mode == SCWP_SYNTH_GATHER_FP16 ||
          ctx->synth_mode == SCWP_SYNTH_SAT))
