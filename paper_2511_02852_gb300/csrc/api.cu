@@ -450,6 +450,12 @@ TileWork tile_bucket_stages(const PatchHost& P) {
 // per item its start and its store (5,000 cycles).
 constexpr double kSatBucketUs = 5.7;
 constexpr double kSatBumpUs = 0.0012;
+// The same for the three-group kernel, of which two CTAs share an SM: weighed
+// with the figures above, its plans were of too few, too long items (a frame
+// of the 1024^2 scene 0.411 ms instead of 0.318).
+constexpr double kSat3BucketUs = 2.0;
+constexpr double kSat3BumpUs = 0.0008;
+constexpr double kSat3Waves = 3.0;     // its patch plans have at least so many waves of items
 constexpr double kSatItemStages = 2.0;
 // The group-sum blend: its launch, and its planes at the rate it reads them
 constexpr double kBlendUs = 3.0;
@@ -459,7 +465,7 @@ constexpr double kBlendBytesPerUs = 6.0e6;
 // reach (grown by a bin) runs before the patch's domain ends: the tiles away
 // from the last columns and rows are one class.  (All terms are multiples of
 // 2^-16 far below 2^37: the differences are exact in float64.)
-TileWork tile_bucket_sat(const PatchHost& P, double* max_passes = nullptr) {
+TileWork tile_bucket_sat(const PatchHost& P, bool three = false, double* max_passes = nullptr) {
     const PatchTablesHost& T = P.T;
     const int ts = synth_sat_tile();
     const int ntx = (T.W + ts - 1) / ts, nty = (T.H + ts - 1) / ts, nb = T.nb;
@@ -480,7 +486,8 @@ TileWork tile_bucket_sat(const PatchHost& P, double* max_passes = nullptr) {
             const double n = dens[i] * ax * ay;
             const double passes = std::max(1.0, std::ceil(n * std::sqrt(n) / (double)P.bk[i].sat_c));
             if (max_passes) *max_passes = std::max(*max_passes, passes);
-            out.est[c * nb + i] = (passes * kSatBucketUs + n * kSatBumpUs) / kStageUs;
+            out.est[c * nb + i] = (three ? passes * kSat3BucketUs + n * kSat3BumpUs
+                                         : passes * kSatBucketUs + n * kSatBumpUs) / kStageUs;
         }
     return out;
 }
@@ -609,23 +616,26 @@ struct ItemRuns {
 // Plan of one patch launched alone: G minimises the simulated makespan over
 // the device's resident CTA slots plus the traffic of the group-sum blend.
 // For the summed-area synthesis, gmul scales the chosen G (the autotuner's
-// search axis), within [1, gcap].
-void plan_patch(PatchHost& P, int slots, bool sat = false, double gmul = 1.0, int gcap = 16) {
-    const TileWork tw = sat ? tile_bucket_sat(P) : tile_bucket_stages(P);
+// search axis), within [1, gcap]; three: for the three-group kernel.
+void plan_patch(PatchHost& P, int slots, bool sat = false, double gmul = 1.0, int gcap = 16, bool three = false) {
+    const TileWork tw = sat ? tile_bucket_sat(P, three) : tile_bucket_stages(P);
     const int nb = P.T.nb;
     int& groups = sat ? P.sat_groups : P.dev.groups_tc;
     const int gmax = std::max(1, std::min(std::min(nb, 16), gcap));
+    int g_lo = 1;
+    if (three)
+        while (g_lo < gmax && (double)tw.tiles * g_lo < kSat3Waves * slots) ++g_lo;
     double best_cost = 0.0;
-    for (int G = 1; G <= gmax; ++G) {
+    for (int G = g_lo; G <= gmax; ++G) {
         ItemRuns r;
         r.add(P.index, tw, G, 1, sat);
-        const double blend = G <= 1 ? 0.0
-                             : sat  ? kBlendUs + (G + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs
-                                    : (G + 1) * 12.0 * P.T.W * P.T.H / kHbmBytesPerUs;
-        if (G > 1 && r.makespan_bound(slots) * kStageUs + blend >= best_cost) continue;
+        const double blend = G <= 1          ? 0.0
+                             : sat && !three ? kBlendUs + (G + 1) * 12.0 * P.T.W * P.T.H / kBlendBytesPerUs
+                                             : (G + 1) * 12.0 * P.T.W * P.T.H / kHbmBytesPerUs;
+        if (G > g_lo && r.makespan_bound(slots) * kStageUs + blend >= best_cost) continue;
         r.sort();
         const double cost = r.makespan(slots) * kStageUs + blend;
-        if (G == 1 || cost < best_cost) {
+        if (G == g_lo || cost < best_cost) {
             best_cost = cost;
             groups = G;
         }
@@ -672,8 +682,9 @@ bool sat3_fits(const PatchHost& P) {
 
 // Plan of all patches in one launch: each patch's G is the smallest that
 // keeps its largest item under `share` of the average per-slot load (a
-// quarter for the tensor-core gather), and all items of all patches run
-// heaviest first.  For the summed-area synthesis the share is the one, of a
+// quarter for the tensor-core gather and the three-group kernel, there no more
+// than the patch's own plan takes), and all items of all patches run heaviest
+// first.  For the nine-plane synthesis the share is the one, of a
 // few, with the smallest modelled makespan and blend: an item's start and
 // store cost nearly half a pass (2.6 of 5.7 us), so a scene that fits one wave
 // of longer items runs them rather than three of single buckets (a quarter for
@@ -681,10 +692,11 @@ bool sat3_fits(const PatchHost& P) {
 void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vector<BlendSpan>& spans,
                   std::vector<double>& item_work_out, bool sat = false) {
     const size_t np = ctx->patches.size();
+    const bool three = sat && ctx->sat_variant == 1;
     std::vector<TileWork> tw(np);
     double total = 0.0;
     for (size_t k = 0; k < np; ++k) {
-        tw[k] = sat ? tile_bucket_sat(*ctx->patches[k]) : tile_bucket_stages(*ctx->patches[k]);
+        tw[k] = sat ? tile_bucket_sat(*ctx->patches[k], three) : tile_bucket_stages(*ctx->patches[k]);
         for (size_t c = 0; c < tw[k].cls.size(); ++c)
             total += (double)tw[k].cls[c].size() * item_work(tw[k], c, 0, 1, sat);
     }
@@ -705,7 +717,8 @@ void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vec
             const int gmax = std::min(std::min(P.T.nb, 16), P.partial_planes);
             int G = 1;
             while (G < gmax && heaviest(k, G) > share * per_slot) ++G;
-            G = std::max(1, std::min(gmax, (int)std::lround(G * gmul)));
+            G = three ? std::max(1, std::min(G, P.sat_groups))
+                      : std::max(1, std::min(gmax, (int)std::lround(G * gmul)));
             // summed-area items: each bucket's passes split over K parts where
             // an item would still outlast the balanced per-slot share of the
             // frame (dense patches whose buckets take many passes)
@@ -733,8 +746,8 @@ void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vec
         }
         return us + (any ? kBlendUs : 0.0);
     };
-    const std::vector<double> shares = sat ? std::vector<double>{4.0, 2.0, 1.4, 1.0, 0.7, 0.5, 0.35, 0.25}
-                                           : std::vector<double>{0.25};
+    const std::vector<double> shares = sat && !three ? std::vector<double>{4.0, 2.0, 1.4, 1.0, 0.7, 0.5, 0.35, 0.25}
+                                                     : std::vector<double>{0.25};
     double share = shares[0], best_cost = 0.0;
     Choice best = choose(share, 1.0), last = best;
     ItemRuns best_runs = runs_of(best);
@@ -757,7 +770,7 @@ void plan_batched(scwp_ctx* ctx, int slots, std::vector<TcItem>& items, std::vec
             share = shares[i];
         }
     }
-    if (sat && ctx->sat_gmul != 1.0) {   // the autotuner's axis
+    if (sat && !three && ctx->sat_gmul != 1.0) {   // the autotuner's axis (in the patches' own plans for three)
         best = choose(share, ctx->sat_gmul);
         best_runs = runs_of(best);
         best_runs.sort();
@@ -1156,13 +1169,13 @@ scwp_status scwp_add_patch(scwp_ctx* ctx, const scwp_patch_desc* desc, int32_t* 
         // can split into parts
         int gpart = std::min(nbmax, 2 * gsat);
         double max_passes = 0.0;
-        const int tiles_sat = tile_bucket_sat(*P, &max_passes).tiles;
+        const int tiles_sat = tile_bucket_sat(*P, false, &max_passes).tiles;
         if (max_passes >= 2.0 && (size_t)64 * 12 * T.W * T.H <= ((size_t)256 << 20)) gpart = 64;
         P->partial_planes = std::max(std::max(D.groups, D.groups_tc), gpart);
         const int variant = (ctx->sat_variant == 1 && P->sat3_ok) ? 1 : 0;
         P->sat_slots = sat_slots_of(variant);
         ctx->sat_slots = P->sat_slots;
-        plan_patch(*P, P->sat_slots, true, ctx->sat_gmul, P->partial_planes);
+        plan_patch(*P, P->sat_slots, true, ctx->sat_gmul, P->partial_planes, variant == 1);
         P->d_items = (TcItem*)dalloc(ctx, P->tc_items.size() * sizeof(TcItem));
         P->d_spans = (BlendSpan*)dalloc(ctx, std::max<size_t>(1, P->tc_spans.size()) * sizeof(BlendSpan));
         P->sat_item_cap = tiles_sat * P->partial_planes;   // G K <= the planes
@@ -1686,7 +1699,7 @@ static scwp_status replan_sat(scwp_ctx* ctx) {
     for (PatchHost* P : ctx->patches) {
         const int variant = (ctx->sat_variant == 1 && P->sat3_ok) ? 1 : 0;
         P->sat_slots = sat_slots_of(variant);
-        plan_patch(*P, P->sat_slots, true, ctx->sat_gmul, P->partial_planes);
+        plan_patch(*P, P->sat_slots, true, ctx->sat_gmul, P->partial_planes, variant == 1);
         if ((int)P->sat_items.size() > P->sat_item_cap) return fail(ctx, SCWP_E_STATE, "summed-area plan capacity");
         CU(cudaMemcpyAsync(P->d_sat_items, P->sat_items.data(), P->sat_items.size() * sizeof(TcItem),
                            cudaMemcpyHostToDevice, ctx->st));

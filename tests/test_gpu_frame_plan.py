@@ -160,6 +160,19 @@ def test_patch_info_describes_the_plan_that_runs(n, side, batched):
     sc.close()
 
 
+def test_three_group_plans_keep_their_waves():
+    """The three-group kernel (two CTAs an SM, one item each) gets at least
+    three waves of items on a patch that has the buckets for it."""
+    from paper_2511_02852_gb300 import scwp
+    sc = scwp.Scene(wl.realistic(), device=0)
+    sc.set_sat_plan(1, 1.0)
+    i = sc.info(0)
+    assert i.sat_variant == 1 and i.sat_items >= 3 * i.sat_slots, (i.sat_items, i.sat_slots)
+    sc.set_sat_plan(0, 1.0)
+    assert sc.info(0).sat_variant == 0
+    sc.close()
+
+
 def scwp_launches(scwp, sc):
     import ctypes
     n = ctypes.c_int64()
